@@ -408,7 +408,14 @@ uint64_t gb_ws_bytes(int64_t slots, int32_t n_aggs) {
 
 // ------------------------------------------------- partitioned variant (P)
 
-constexpr uint32_t PART_MAX_GRID = 512;  // CTAs of the histogram / scatter passes
+constexpr uint32_t PART_HIST_COLS = 512;                 // columns of the histogram
+constexpr uint32_t PART_MAX_GRID = PART_HIST_COLS - 1;  // CTAs of the histogram / scatter passes
+                                                        // (the last column holds part_extra)
+
+// With at most 2^PART_SPLIT_BITS partitions the aggregation pass cuts the
+// records into equal pieces instead of taking whole partitions: 256
+// partitions would occupy 256 of its ~600 CTAs.
+constexpr int PART_SPLIT_BITS = 8;
 
 bool part_shape(int shape) {
   return shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
@@ -428,7 +435,7 @@ PartLayout part_layout(int64_t slots, int32_t n_aggs, int bits, int64_t n_rows) 
   const uint64_t P = 1ull << bits;
   const uint64_t bins = 1ull << PART_L1_BITS;
   L.hist = align_up(gb_ws_bytes(slots, n_aggs), 256);
-  L.starts = align_up(L.hist + 4ull * P * PART_MAX_GRID, 256);
+  L.starts = align_up(L.hist + 4ull * P * PART_HIST_COLS, 256);
   L.cursor = align_up(L.starts + 8ull * (P + 1), 256);
   L.cursor1 = align_up(L.cursor + 4ull * P, 256);
   L.l2_tiles = align_up(L.cursor1 + 4ull * bins, 256);
@@ -459,11 +466,20 @@ rel_status run_partitioned(GbParams& p, const rel_plan* plan, int shape, const G
   p.cursor = (unsigned int*)(base + L.cursor);
   p.cursor1 = (unsigned int*)(base + L.cursor1);
   p.l2_tiles = (unsigned int*)(base + L.l2_tiles);
+  p.part_extra = (unsigned int*)p.hist + ((size_t)PART_MAX_GRID << p.part_bits);
   p.recs = (PartRec*)(base + L.recs);
   p.recs1 = p.part_bits > PART_L1_BITS ? (PartRec*)(base + L.recs1) : nullptr;
+  p.part_split = plan->part_bits <= PART_SPLIT_BITS &&
+                 plan->slots >= (int64_t)plan->smem_slots << plan->part_bits;
   uint32_t grid = 2u * (uint32_t)relhost::device_sms();
   p.fixed_grid = grid > PART_MAX_GRID ? PART_MAX_GRID : grid;
-  const uint32_t agg_slots = p.smem_slots;
+  // Tables of the aggregation pass.  At the planned load (up to 1/2) one row
+  // in ten leaves its home bucket; twice the slots make that one in 25, which
+  // pays where a partition has the records to make up for the slots it scans
+  // (1e8 uniform rows, 2e6 groups, 24K records a partition: 0.83 -> 0.62 ms;
+  // 2e8 Zipf rows, 9K: 1.01 -> 1.16 ms)
+  uint32_t agg_slots = p.smem_slots;
+  if (agg_slots <= 1024 && p.n_rows >> p.part_bits >= 16384) agg_slots *= 2;
   p.smem_slots = 0;  // passes 1-2 keep only the pinned thread-private layer
   if (!p.tiny_frozen) {
     p.tiny_slots = 0;
@@ -517,6 +533,8 @@ void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
   // (more keys per partition than half a table of the largest size)
   uint64_t spill = (uint64_t)est / 4;
   if (2 * keys_per_part > (uint64_t)plan->smem_slots) spill = 2 * (uint64_t)est;
+  // few partitions: their pieces meet in the global table (part_split)
+  if (bits <= PART_SPLIT_BITS) spill = std::max(spill, (uint64_t)plan->smem_slots << bits);
   plan->slots = (int64_t)next_pow2(spill > 65536 ? spill : 65536);
   (void)n_rows;
 }
@@ -534,10 +552,11 @@ void choose_layers(int64_t est, int words, rel_plan* plan) {
   } else if (est <= 24 && words <= 2) {
     plan->variant = REL_VAR_SMEM;
     plan->tiny_slots = 32;
-  } else if (est <= 2048) {
+  } else if (est <= (words == 2 ? 4096 : 2048)) {
     plan->variant = REL_VAR_SMEM;
     plan->tiny_slots = words <= 6 ? 8 : 0;  // catches a skewed input's hottest keys
     plan->smem_slots = (int32_t)next_pow2((uint64_t)(2 * est));
+    if (plan->smem_slots > SHARED_MAX_SLOTS) plan->smem_slots = SHARED_MAX_SLOTS;
   } else {
     plan->variant = REL_VAR_GLOBAL;
     plan->tiny_slots = words <= 6 ? 8 : 0;

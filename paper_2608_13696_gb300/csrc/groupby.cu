@@ -21,6 +21,7 @@
 // occupied slots into dense output rows (warp ballot / popc, one atomic per
 // warp).  MODE_KEYSET counts distinct keys instead (the exact sizing pass).
 #include "groupby.cuh"
+#include "smtab.cuh"
 
 namespace rel {
 
@@ -249,9 +250,9 @@ __device__ __forceinline__ void red_words(const GbParams& p, unsigned long long*
   for (int a = 0; a < S::A; ++a) {
     if (live_agg<S>(p, a)) {
       if (is_umax<S>(p, a))
-        atomicMax(w + a, (unsigned long long)x.v[a]);
+        redg_max(w + a, x.v[a]);
       else
-        atomicAdd(w + a, (unsigned long long)x.v[a]);
+        redg_add(w + a, x.v[a]);
     }
   }
 }
@@ -259,34 +260,17 @@ __device__ __forceinline__ void red_words(const GbParams& p, unsigned long long*
 // Shared-memory words: a MIN / MAX word is read first and only raised by an
 // atomic when the row improves it -- under skew most rows of a hot key do not,
 // so most of those atomics (and their serialisation on one address) vanish.
-template <class S, bool COUNT32 = false>
+template <class S>
 __device__ __forceinline__ void red_words_smem(const GbParams& p, unsigned long long* w,
                                                const Vals<S::A>& x) {
-  if constexpr (COUNT32 && !S::RT && S::A == 4) {
-    // (sum, count, min, max) of a 32-byte slot: the MIN / MAX pair is read
-    // with one 16-byte load (w is 32-byte aligned)
-    sadd64(w, x.v[0]);
-    atomicAdd((unsigned int*)(w + 1), (unsigned int)x.v[1]);
-    unsigned long long mn, mx;
-    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];"
-                 : "=l"(mn), "=l"(mx)
-                 : "r"(smem_u32(w + 2)));
-    if ((unsigned long long)x.v[2] > mn) atomicMax(w + 2, (unsigned long long)x.v[2]);
-    if ((unsigned long long)x.v[3] > mx) atomicMax(w + 3, (unsigned long long)x.v[3]);
-  } else {
 #pragma unroll
-    for (int a = 0; a < S::A; ++a) {
-      if (live_agg<S>(p, a)) {
-        if (COUNT32 && a == 1) {
-          // key/value shapes: word 1 counts rows; below 2^32 rows per table
-          // (a partitioned input has fewer) a 32-bit add on its low half is exact
-          atomicAdd((unsigned int*)(w + 1), (unsigned int)x.v[1]);
-        } else if (is_umax<S>(p, a)) {
-          if ((unsigned long long)x.v[a] > *(volatile unsigned long long*)(w + a))
-            atomicMax(w + a, (unsigned long long)x.v[a]);
-        } else {
-          sadd64(w + a, x.v[a]);
-        }
+  for (int a = 0; a < S::A; ++a) {
+    if (live_agg<S>(p, a)) {
+      if (is_umax<S>(p, a)) {
+        if ((unsigned long long)x.v[a] > *(volatile unsigned long long*)(w + a))
+          atomicMax(w + a, (unsigned long long)x.v[a]);
+      } else {
+        sadd64(w + a, x.v[a]);
       }
     }
   }
@@ -322,6 +306,15 @@ __device__ __forceinline__ bool gtab_update_inl(const GbParams& p, uint64_t ek,
 template <class S>
 __device__ __forceinline__ bool gtab_update(const GbParams& p, uint64_t ek, const Vals<S::A>& x) {
   return gtab_update_inl<S>(p, ek, x);
+}
+
+// One key/value row into the global table, out of line (the rare path of a
+// kernel whose registers are better spent elsewhere).
+template <class S>
+__device__ __noinline__ void gtab_row(const GbParams& p, uint64_t ek, uint64_t val) {
+  Vals<S::A> x;
+  S::from_val(val, x);
+  gtab_update_inl<S>(p, ek, x);
 }
 
 // Key set for the exact distinct count; false when the set overflowed.
@@ -936,166 +929,283 @@ __global__ void __launch_bounds__(256) gb_part_sum(const __grid_constant__ GbPar
   if (lane == 0) p.part_start[part] = s;
 }
 
+// Records a piece of an oversized partition holds: partitions above this (four
+// times the average, as skewed keys make) are cut into pieces of about it.
+__device__ __forceinline__ unsigned long long part_piece(unsigned long long total, uint32_t P) {
+  const unsigned long long four = 4 * (total / P);
+  return four > 4096 ? four : 4096;
+}
+
 // partition totals -> first record of each partition; part_start[P] = all.
-// Also the cursors of both scatter levels and the level-2 pass's tiles.
+// Also the cursors of both scatter levels, the level-2 pass's tiles, and the
+// list of the second and further pieces of oversized partitions (part_extra:
+// their number, then partition | piece << PART_MAX_BITS; at most P / 4 of
+// them).  One CTA, so its memory requests bound it: the totals go through
+// shared memory (padded; counts and positions are 32-bit), read and written
+// in order by consecutive threads instead of 128 bytes apart (16384
+// partitions: 39 -> 18 us).
+__device__ __forceinline__ uint32_t scan_pad(uint32_t i) { return i + (i >> 5); }
+
 __global__ void __launch_bounds__(1024) gb_part_scan2(const __grid_constant__ GbParams p) {
-  __shared__ unsigned long long total, tiles_total;
-  const uint32_t P = 1u << p.part_bits;
-  const uint32_t per = (P + blockDim.x - 1) / blockDim.x;
-  const uint32_t b = threadIdx.x * per, e = b + per < P ? b + per : P;
-  unsigned long long s = 0;
-  for (uint32_t i = b; i < e; ++i) s += p.part_start[i];
-  unsigned long long run = block_exclusive_scan(s, &total);
-  for (uint32_t i = b; i < e; ++i) {
-    const unsigned long long v = p.part_start[i];
-    p.part_start[i] = run;
-    p.cursor[i] = (unsigned int)run;
-    run += v;
-  }
-  if (threadIdx.x == 0) p.part_start[P] = total;
+  extern __shared__ uint32_t cnt[];  // [scan_pad(P)] totals, then first records
+  __shared__ unsigned long long total, tiles_total, extra_total;
+  const uint32_t P = 1u << p.part_bits, tid = threadIdx.x;
+  for (uint32_t i = tid; i < P; i += 1024) cnt[scan_pad(i)] = (uint32_t)p.part_start[i];
   __syncthreads();
+  const uint32_t per = (P + 1023) / 1024;
+  const uint32_t b = tid * per, e = b + per < P ? b + per : P;
+  unsigned long long s = 0;
+  for (uint32_t i = b; i < e; ++i) s += cnt[scan_pad(i)];
+  unsigned long long run = block_exclusive_scan(s, &total);
+  const unsigned long long piece = part_piece(total, P);
+  uint32_t extra = 0;
+  for (uint32_t i = b; i < e; ++i) {
+    const uint32_t v = cnt[scan_pad(i)];
+    if (v > piece) extra += (uint32_t)((v - 1) / piece);
+  }
+  uint32_t at = (uint32_t)block_exclusive_scan(extra, &extra_total);
+  for (uint32_t i = b; i < e; ++i) {
+    const uint32_t v = cnt[scan_pad(i)];
+    cnt[scan_pad(i)] = (uint32_t)run;
+    run += v;
+    if (v <= piece) continue;
+    const uint32_t n = (uint32_t)((v - 1) / piece);
+    for (uint32_t c = 1; c <= n; ++c) p.part_extra[1 + at++] = i | c << PART_MAX_BITS;
+  }
+  if (tid == 0) {
+    p.part_start[P] = total;
+    p.part_extra[0] = (uint32_t)extra_total;
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < P; i += 1024) {
+    const uint32_t v = cnt[scan_pad(i)];
+    p.part_start[i] = v;
+    p.cursor[i] = v;
+  }
   // level-1 bins: 2^shift1 consecutive partitions each
   const uint32_t shift1 = p.part_bits > PART_L1_BITS ? p.part_bits - PART_L1_BITS : 0;
   const uint32_t B1 = P >> shift1;
   unsigned long long tiles = 0;
-  if (threadIdx.x < B1) {
-    const unsigned long long s1 = p.part_start[threadIdx.x << shift1];
-    const unsigned long long e1 = p.part_start[(threadIdx.x + 1) << shift1];
-    p.cursor1[threadIdx.x] = (unsigned int)s1;
+  if (tid < B1) {
+    const uint32_t s1 = cnt[scan_pad(tid << shift1)];
+    const unsigned long long e1 = tid + 1 < B1 ? cnt[scan_pad((tid + 1) << shift1)] : total;
+    p.cursor1[tid] = s1;
     tiles = (e1 - s1 + PART_TILE - 1) / PART_TILE;
   }
   const unsigned long long tp = block_exclusive_scan(tiles, &tiles_total);
-  if (threadIdx.x < B1) p.l2_tiles[threadIdx.x] = (unsigned int)tp;
-  if (threadIdx.x == 0) p.l2_tiles[B1] = (unsigned int)tiles_total;
+  if (tid < B1) p.l2_tiles[tid] = (unsigned int)tp;
+  if (tid == 0) p.l2_tiles[B1] = (unsigned int)tiles_total;
 }
 
-// Insert-or-accumulate into a partition's shared-memory table; a key that
-// finds no slot within 32 probes goes to the global table and marks the
-// partition as spilled.
-template <class S>
-__device__ __forceinline__ void part_insert(const GbParams& p, uint64_t* tk, unsigned long long* ta,
-                                            uint32_t TS, uint64_t ek, const Vals<S::A>& x,
-                                            int* ovf) {
-  uint32_t s = small_slot_of(ek, TS - 1, SHARED_MULT);
-  for (uint32_t k = 0; k < 32; ++k) {
-    uint64_t cur = *(volatile uint64_t*)(tk + s);
-    if (cur == 0) {
-      cur = atomicCAS((unsigned long long*)(tk + s), 0ull, (unsigned long long)ek);
-      if (cur == 0) cur = ek;
-    }
-    if (cur == ek) {
-      red_words_smem<S, true>(p, ta + (size_t)s * S::A, x);
-      return;
-    }
-    s = (s + 1) & (TS - 1);
-  }
-  *(volatile int*)ovf = 1;
-  gtab_update<S>(p, ek, x);
-}
-
-// record groups in flight per warp in the aggregation pass (2, 4, 8: 1.36, 1.40
-// and 1.94 ms on 2e8 Zipf rows: fewer registers, more warps)
+// record groups in flight per warp in the aggregation pass (2 and 4: 1.01 and
+// 1.13 ms on 2e8 Zipf(1.1) rows, equal on uniform keys)
 constexpr int PA_R = 2;
 
-// Pass 3: each CTA aggregates whole partitions in a shared-memory table of
-// p.smem_slots slots and writes their groups straight to the output (warp
-// ballot / popc, one atomic per warp).  Every key lives in one partition, so
-// no group is emitted twice -- unless the table overflows: then the whole
-// partition is merged into the global table instead, which the compaction
-// kernel emits afterwards.
-template <class S>
-__global__ void __launch_bounds__(GB_BLOCK) gb_part_agg(const __grid_constant__ GbParams p,
-                                                         const __grid_constant__ GbOut o) {
-  constexpr int A = S::A;
+// The key that most lanes of the warp hold, 0 when none is held by four.
+__device__ __forceinline__ uint64_t frequent_key(uint64_t ek) {
+  const unsigned same = __match_any_sync(0xffffffffu, (unsigned long long)ek);
+  const int n = ek ? __popc(same) : 0;
+  const unsigned best = __reduce_max_sync(0xffffffffu, (unsigned)n);
+  const int lane = __ffs(__ballot_sync(0xffffffffu, (unsigned)n == best)) - 1;
+  const uint64_t k = __shfl_sync(0xffffffffu, ek, lane);
+  return best >= 4 ? k : 0;
+}
+
+// Pass 3: CTAs aggregate partitions in a shared-memory table of p.smem_slots
+// slots and write their groups straight to the output (warp ballot / popc, one
+// atomic per warp and partition).  Every key lives in one partition, so no
+// group is emitted twice -- unless a CTA saw only a piece of the partition or
+// its table overflowed: then what it holds goes to the global table instead,
+// which the compaction kernel emits afterwards.
+//
+// Two ways to share the records out:
+//  * whole partitions, CTA after CTA, then the further pieces of oversized
+//    ones (part_extra);
+//  * p.part_split: equal pieces of the record array, one per CTA, whatever
+//    partitions they touch.  For plans with fewer partitions than CTAs, whose
+//    whole partitions would leave most SMs idle (1e8 rows, 4000 groups, 16
+//    partitions: 16.8 ms in 16 CTAs).  The host sets it when the global table
+//    has a slot for every slot of the partition tables.
+template <int NA>
+__global__ void __launch_bounds__(GB_BLOCK, 4) gb_part_agg(const __grid_constant__ GbParams p,
+                                                           const __grid_constant__ GbOut o) {
+  using S = ShapeKV<int64_t, NA>;
   extern __shared__ __align__(16) uint8_t sm[];
-  __shared__ int ovf;
+  __shared__ int ovf[2];  // of this piece and the next
   const uint32_t TS = p.smem_slots;
-  uint64_t* tk = (uint64_t*)sm;
-  unsigned long long* ta = (unsigned long long*)(tk + TS);
+  SmTab<NA> t;
+  t.bind(sm, TS);
+  t.clear();
+  if (threadIdx.x < 2) ovf[threadIdx.x] = 0;
   const uint32_t P = 1u << p.part_bits;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  // a partition far above the average (skewed keys) is split into up to
-  // PART_CHUNKS chunks on different CTAs, which then merge into the global
-  // table instead of emitting
-  const unsigned long long avg = p.part_start[P] / P;
-  const unsigned long long chunk_min = 4 * avg > 4096 ? 4 * avg : 4096;
-  for (uint32_t item = blockIdx.x; item < P * PART_CHUNKS; item += gridDim.x) {
-    // chunk-major numbering: the first chunks of all partitions come first and
-    // spread over every CTA
-    const uint32_t part = item % P, c = item / P;
-    const unsigned long long pb = p.part_start[part], pe = p.part_start[part + 1];
-    const unsigned long long size = pe - pb;
-    unsigned long long nch = (size + chunk_min - 1) / chunk_min;
-    nch = nch < 1 ? 1 : (nch > PART_CHUNKS ? PART_CHUNKS : nch);
-    if (c >= nch) continue;  // uniform across the CTA
-    const unsigned long long beg = pb + size * c / nch, end = pb + size * (c + 1) / nch;
-    for (uint32_t i = threadIdx.x; i < TS * (1 + A); i += GB_BLOCK) tk[i] = 0;
-    if (threadIdx.x == 0) ovf = nch > 1;
-    __syncthreads();
-    {
-      // each warp takes 32 consecutive records at a time, PA_R such groups
-      // loaded before any is used, and the next PA_R groups' loads go out
-      // before this batch is inserted (the pass waits on load latency).  Lanes
-      // of one key are not combined in registers first: on the partitions of
-      // skewed keys that did not cost less than the serialised shared-memory
-      // atomics it saves (2e8 Zipf(1.1) rows: 2.0 -> 1.9 ms without it)
-      const int warp = threadIdx.x >> 5;
-      const unsigned long long bstep = (unsigned long long)GB_BLOCK * PA_R;
-      longlong2 rec[PA_R];
-      unsigned long long b00 = beg + (unsigned long long)warp * 32 * PA_R;
-#pragma unroll
-      for (int rr = 0; rr < PA_R; ++rr) {
-        const unsigned long long i = b00 + (unsigned long long)rr * 32 + lane;
-        rec[rr] = i < end ? __ldcs((const longlong2*)(p.recs + i)) : make_longlong2(0, 0);
-      }
-      for (; b00 < end; b00 += bstep) {
-        // the next groups' records go out before this group's are inserted
-        longlong2 nxt[PA_R];
-#pragma unroll
-        for (int rr = 0; rr < PA_R; ++rr) {
-          const unsigned long long i = b00 + bstep + (unsigned long long)rr * 32 + lane;
-          nxt[rr] = i < end ? __ldcs((const longlong2*)(p.recs + i)) : make_longlong2(0, 0);
-        }
-#pragma unroll
-        for (int rr = 0; rr < PA_R; ++rr) {
-          if (b00 + (unsigned long long)rr * 32 + lane >= end) continue;
-          Vals<A> x;
-          S::from_val((uint64_t)rec[rr].y, x);
-          part_insert<S>(p, tk, ta, TS, (uint64_t)rec[rr].x, x, &ovf);
-        }
-#pragma unroll
-        for (int rr = 0; rr < PA_R; ++rr) rec[rr] = nxt[rr];
-      }
+  const unsigned long long total = p.part_start[P];
+  const unsigned long long piece = part_piece(total, P);
+  const uint32_t items = P + (p.part_split ? 0 : p.part_extra[0]);
+  // this CTA's piece of the record array (part_split)
+  const unsigned long long even = (total + gridDim.x - 1) / gridDim.x;
+  const unsigned long long per = even > 1024 ? even : 1024;
+  const unsigned long long piece0 = p.part_split ? per * blockIdx.x : 0;
+  const unsigned long long piece1 = p.part_split && piece0 + per < total ? piece0 + per : total;
+
+  // next piece of work from item on: records [beg, end), all of a partition or not
+  uint32_t item = blockIdx.x;
+  unsigned long long beg = 0, end = 0;
+  bool whole = true;
+  auto next = [&]() -> bool {
+    if (p.part_split) {
+      if (end >= piece1) return false;
+      beg = end;
+      while (p.part_start[item + 1] <= beg) ++item;
+      const unsigned long long pb = p.part_start[item], pe = p.part_start[item + 1];
+      end = pe < piece1 ? pe : piece1;
+      whole = beg == pb && end == pe;
+      return true;
     }
+    for (; item < items; item += gridDim.x) {
+      const uint32_t x = item < P ? item : p.part_extra[1 + item - P];
+      const uint32_t part = x & ((1u << PART_MAX_BITS) - 1), c = x >> PART_MAX_BITS;
+      const unsigned long long pb = p.part_start[part], pe = p.part_start[part + 1];
+      const unsigned long long size = pe - pb;
+      if (size == 0) continue;  // uniform across the CTA
+      const unsigned long long nch = (size - 1) / piece + 1;
+      beg = pb + size * c / nch;
+      end = pb + size * (c + 1) / nch;
+      whole = nch == 1;
+      item += gridDim.x;
+      return true;
+    }
+    return false;
+  };
+  if (p.part_split) {
+    if (piece0 >= piece1) return;
+    uint32_t lo = 0, hi = P;  // part_start[lo] <= piece0 < part_start[hi]
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (p.part_start[mid] <= piece0) lo = mid; else hi = mid;
+    }
+    item = lo;
+    end = piece0;
+  }
+
+  // A warp takes PA_R groups of 32 consecutive records at a time; the next
+  // batch's loads go out before this batch is inserted, the next piece's first
+  // ones before this piece's groups are written out.  (32-bit offsets inside a
+  // piece: pieces are a fraction of fewer than 2^32 records.)
+  constexpr uint32_t STEP = GB_BLOCK * PA_R;
+  longlong2 rec[PA_R];
+  const longlong2* src = nullptr;  // this lane's first record of the piece
+  uint32_t off = 0, len = 0;       // of the warp's next batch; of the piece
+  auto load = [&](longlong2(&r)[PA_R], uint32_t at) {
+#pragma unroll
+    for (int q = 0; q < PA_R; ++q)
+      r[q] = at + q * 32 + lane < len ? __ldcs(src + at + q * 32) : make_longlong2(0, 0);
+  };
+  auto start = [&]() {
+    src = (const longlong2*)(p.recs + beg) + lane;
+    len = (uint32_t)(end - beg);
+    off = warp * 32 * PA_R;
+    load(rec, off);
+  };
+  bool more = next();
+  if (more) start();
+  __syncthreads();
+  for (int turn = 0; more; turn ^= 1) {
+    uint64_t hot = 0, hw[NA];  // the key in registers (0: none) and its words
+    if (!whole) hot = frequent_key((uint64_t)rec[0].x);
+#pragma unroll
+    for (int a = 0; a < NA; ++a) hw[a] = 0;
+    for (; off < len; off += STEP) {
+      uint64_t ek[PA_R], val[PA_R];
+      uint32_t slot[PA_R];
+#pragma unroll
+      for (int q = 0; q < PA_R; ++q) {
+        ek[q] = (uint64_t)rec[q].x;  // 0 past the end: a record's key is not 0
+        val[q] = (uint64_t)rec[q].y;
+      }
+      load(rec, off + STEP);
+      if (hot) {  // uniform across the warp
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < PA_R; ++q) {
+          if (ek[q] == hot) {
+            ek[q] = 0;
+            hw[0] += val[q];
+            hw[1] += 1;
+            if constexpr (NA == 4) {
+              const uint64_t mn = val[q] ^ MIN_FLIP, mx = val[q] ^ MAX_FLIP;
+              hw[2] = hw[2] > mn ? hw[2] : mn;
+              hw[3] = hw[3] > mx ? hw[3] : mx;
+            }
+          }
+          any |= ek[q] != 0;
+        }
+        if (!__any_sync(0xffffffffu, any)) continue;
+      }
+      const uint32_t left = t.find(ek, 32, slot);
+      if (left) {
+        *(volatile int*)(ovf + turn) = 1;
+#pragma unroll
+        for (int q = 0; q < PA_R; ++q)
+          if (left >> q & 1) gtab_row<S>(p, ek[q], val[q]);
+      }
+      __syncwarp();
+      t.add(slot, val);
+    }
+    if (hot) {  // a piece goes to the global table anyway
+      Vals<NA> x;
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        uint64_t w = hw[a];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+          const uint64_t y = __shfl_xor_sync(0xffffffffu, w, o);
+          w = a < 2 ? w + y : (w > y ? w : y);
+        }
+        x.v[a] = w;
+      }
+      if (lane == 0) gtab_update_inl<S>(p, hot, x);
+    }
+    const bool direct = whole;
+    more = next();
+    if (more) start();
     __syncthreads();
-    const bool spill = ovf != 0;
-    for (uint32_t base = 0; base < TS; base += GB_BLOCK) {
-      const uint32_t s = base + threadIdx.x;
-      const uint64_t ek = s < TS ? tk[s] : 0;
-      const bool occ = ek != 0;
-      if (spill) {  // partition did not fit: everything to the global table
-        if (occ) {
-          Vals<A> x;
-#pragma unroll
-          for (int a = 0; a < A; ++a) x.v[a] = ta[(size_t)s * A + a];
-          gtab_update<S>(p, ek, x);
-        }
-        continue;
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, occ);
-      if (!m) continue;
-      unsigned long long wb = 0;
-      if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)__popc(m));
+    const bool spill = !direct || ovf[turn] != 0;
+    if (threadIdx.x == 0) ovf[turn ^ 1] = 0;
+    // each warp owns a stretch of the slots: one output claim for all of it
+    const uint32_t W = TS / (GB_BLOCK / 32), s0 = warp * W;
+    unsigned long long wb = 0;
+    if (!spill) {
+      uint32_t n = 0;
+      for (uint32_t i = lane; i < W; i += 32) n += t.key_of(s0 + i) != 0;
+      n = __reduce_add_sync(0xffffffffu, n);
+      if (lane == 0 && n) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)n);
       wb = __shfl_sync(0xffffffffu, wb, 0);
+    }
+    for (uint32_t i = lane; i < W; i += 32) {
+      const uint64_t ek = t.key_of(s0 + i);
+      const bool occ = ek != 0;
+      const unsigned m = __ballot_sync(0xffffffffu, occ);
       if (occ) {
-        const uint64_t pos = wb + __popc(m & lt);
-        if (pos < (uint64_t)o.capacity) {
-          o.keys[pos] = (int64_t)(ek ^ KEY_FLIP);
+        uint64_t w[NA];
+        t.words(s0 + i, w);
+        t.clear_slot(s0 + i);  // ready for the next piece
+        if (spill) {  // a piece, or a partition that did not fit
+          Vals<NA> x;
 #pragma unroll
-          for (int a = 0; a < A; ++a) o.aggs[a][pos] = agg_decode(p.aop[a], ta[(size_t)s * A + a]);
+          for (int a = 0; a < NA; ++a) x.v[a] = w[a];
+          gtab_update<S>(p, ek, x);
+        } else {
+          const uint64_t pos = wb + __popc(m & lt);
+          if (pos < (uint64_t)o.capacity) {
+            o.keys[pos] = (int64_t)(ek ^ KEY_FLIP);
+#pragma unroll
+            for (int a = 0; a < NA; ++a) o.aggs[a][pos] = agg_decode(p.aop[a], w[a]);
+          }
         }
       }
+      wb += __popc(m);
     }
     __syncthreads();
   }
@@ -1289,32 +1399,42 @@ rel_status gb_launch_part_scan(const GbParams& p, bool cta_offsets, cudaStream_t
   else
     gb_part_sum<<<(P + 7) / 8, 256, 0, st>>>(p);
   relhost::launch_end(relhost::K_GB_PSCAN, st);
+  const int smem = (int)(4 * (P + P / 32));
+  const cudaError_t e0 =
+      cudaFuncSetAttribute(gb_part_scan2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e0 != cudaSuccess) return relhost::cuda_fail(e0, "cudaFuncSetAttribute(partition scan)");
   relhost::launch_begin(relhost::K_GB_PSCAN, st);
-  gb_part_scan2<<<1, 1024, 0, st>>>(p);
+  gb_part_scan2<<<1, 1024, smem, st>>>(p);
   relhost::launch_end(relhost::K_GB_PSCAN, st);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(partition scan)");
 }
 
+namespace {
+
+template <int NA>
+rel_status launch_part_agg(const GbParams& p, const GbOut& o, cudaStream_t st) {
+  auto kern = gb_part_agg<NA>;
+  const size_t smem = SmTab<NA>::bytes(p.smem_slots);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(partition agg)");
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GB_BLOCK, smem);
+  if (e != cudaSuccess || per_sm < 1) return relhost::cuda_fail(e, "occupancy(partition agg)");
+  const uint32_t P = 1u << p.part_bits;
+  uint32_t grid = (uint32_t)relhost::device_sms() * (uint32_t)per_sm;
+  if (!p.part_split && grid > P) grid = P;  // + the further pieces of a few partitions
+  relhost::launch_begin(relhost::K_GB_PAGG, st);
+  kern<<<grid, GB_BLOCK, smem, st>>>(p, o);
+  relhost::launch_end(relhost::K_GB_PAGG, st);
+  e = cudaGetLastError();
+  return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(partition agg)");
+}
+
+}  // namespace
+
 rel_status gb_launch_part_agg(const GbParams& p, int shape, const GbOut& o, cudaStream_t st) {
-  return with_part_shape(shape, [&](auto s) -> rel_status {
-    using S = decltype(s);
-    auto kern = gb_part_agg<S>;
-    const size_t smem = 8ull * p.smem_slots * (1 + S::A);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(partition agg)");
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GB_BLOCK, smem);
-    if (e != cudaSuccess || per_sm < 1) return relhost::cuda_fail(e, "occupancy(partition agg)");
-    const uint32_t P = 1u << p.part_bits;
-    uint32_t grid = (uint32_t)relhost::device_sms() * (uint32_t)per_sm;
-    if (grid > P) grid = P;
-    relhost::launch_begin(relhost::K_GB_PAGG, st);
-    kern<<<grid, GB_BLOCK, smem, st>>>(p, o);
-    relhost::launch_end(relhost::K_GB_PAGG, st);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(partition agg)");
-  });
+  return gb_shape_width(shape) == 4 ? launch_part_agg<4>(p, o, st) : launch_part_agg<2>(p, o, st);
 }
 
 rel_status gb_launch_compact(const GbParams& p, const GbOut& o, cudaStream_t st) {

@@ -30,7 +30,6 @@ struct alignas(16) PartRec {
   long long val;
 };
 constexpr int PART_MAX_BITS = 14;  // at most 16384 partitions
-constexpr int PART_CHUNKS = 16;    // CTAs that may share one oversized partition
 // Streaming scatter in two levels: the first writes records into at most
 // 2^PART_L1_BITS bins (the top bits of the partition index), the second
 // splits every bin into its partitions.  Both sort a tile of PART_TILE
@@ -94,6 +93,7 @@ struct GbParams {
   int32_t req_tile, req_stages;  // staging chosen by the plan (0: automatic)
   // partitioned variant
   uint32_t part_bits;       // log2 of the partition count
+  uint32_t part_split;      // aggregation: equal pieces of the records, not whole partitions
   uint32_t fixed_grid;      // CTAs of the histogram and scatter passes (equal)
   uint32_t* hist;           // [P][fixed_grid] counts, then exclusive offsets
   unsigned long long* part_start;  // [P + 1] first record of each partition
@@ -101,6 +101,7 @@ struct GbParams {
   PartRec* recs1;           // streaming, part_bits > PART_L1_BITS: records by level-1 bin
   unsigned int* cursor;     // [P] next free record of each partition
   unsigned int* cursor1;    // [2^PART_L1_BITS] next free record of each level-1 bin
+  unsigned int* part_extra; // further pieces of oversized partitions (gb_part_scan2)
   unsigned int* l2_tiles;   // [bins + 1] exclusive prefix of the level-2 tiles per bin
   // global table (or key set in MODE_KEYSET)
   uint64_t* tkeys;

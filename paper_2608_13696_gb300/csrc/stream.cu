@@ -11,14 +11,14 @@
 //  * pinned hot keys (from the sample sketch): a one-probe perfect-hash test
 //    against the pinned key, then thread-private accumulators in shared
 //    memory (one column per thread: no atomics, no bank conflicts);
-//  * optionally a CTA-shared table with shared-memory atomics;
 //  * the global table: every row still unplaced issues its first slot read
 //    before any is resolved (ST_U independent L2 round trips per thread),
 //    then claims or accumulates with CAS / RED atomics, bounded probing.
 // At the end each CTA folds its thread-private words (warp shuffles, then
-// shared atomics) and its shared table into the global table, which the
-// compaction kernel turns into the output.
+// shared atomics) into the global table, which the compaction kernel turns
+// into the output.  Plans with CTA-shared slots run gb_smem_k instead.
 #include "groupby.cuh"
+#include "smtab.cuh"
 
 namespace rel {
 
@@ -32,7 +32,6 @@ constexpr int pin_max() {
   return NA == 4 ? 8 : 16;
 }
 constexpr int ST_PIN_LIMIT = 16;
-constexpr uint32_t ST_SMEM_MULT = 0x85EBCA77u;
 
 template <int NA>
 __device__ __forceinline__ void words_of(uint64_t v, uint64_t (&w)[NA]) {
@@ -55,9 +54,9 @@ __device__ __forceinline__ void red_global(unsigned long long* t, const uint64_t
 #pragma unroll
   for (int a = 0; a < NA; ++a) {
     if (umax_word<NA>(a))
-      atomicMax(t + a, (unsigned long long)w[a]);
+      redg_max(t + a, w[a]);
     else
-      atomicAdd(t + a, (unsigned long long)w[a]);
+      redg_add(t + a, w[a]);
   }
 }
 
@@ -108,20 +107,18 @@ struct KeyPair<int32_t> {
   }
 };
 
-template <class KT, int NA, bool PIN, bool SMT>
+template <class KT, int NA, bool PIN>
 __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant__ GbParams p) {
   extern __shared__ __align__(16) uint8_t sm[];
   // [pinned keys by slot: 32 x 8 B][dense id by slot: 32 B][key by dense id:
   //  16 x 8 B][CTA sums: 16 x 4 x 8 B][thread-private words: PM x NA x
-  //  ST_BLOCK x 8 B][shared table keys: S x 8 B][shared table words: S x NA x 8 B]
+  //  ST_BLOCK x 8 B]
   constexpr int PM = pin_max<NA>();
   uint64_t* pk = (uint64_t*)sm;
   uint8_t* dense = sm + 256;
   uint64_t* pkd = (uint64_t*)(sm + 288);
   unsigned long long* csum = (unsigned long long*)(sm + 416);
   uint64_t* acc = (uint64_t*)(sm + 416 + 8 * ST_PIN_LIMIT * 4);
-  uint64_t* sk = acc + (PIN ? PM * NA * ST_BLOCK : 0);
-  unsigned long long* sa = (unsigned long long*)(sk + (SMT ? p.smem_slots : 0));
   const int tid = threadIdx.x;
   const uint32_t tmask = p.tiny_slots - 1;
 
@@ -137,8 +134,6 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
     for (int i = tid; i < PM * NA * ST_BLOCK; i += ST_BLOCK) acc[i] = 0;
     for (int i = tid; i < PM * NA; i += ST_BLOCK) csum[i] = 0;
   }
-  if (SMT)
-    for (uint32_t i = tid; i < p.smem_slots * (1 + NA); i += ST_BLOCK) sk[i] = 0;
   __syncthreads();
 
   const KT* keys = (const KT*)p.col[p.key_col[0]];
@@ -200,33 +195,6 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
         red_global<NA>(p.hdr->side_aggs, w);
         continue;
       }
-      if (SMT) {
-        uint32_t s = small_slot_of(ek[j], p.smem_slots - 1, ST_SMEM_MULT);
-        bool placed = false;
-        for (uint32_t i = 0; i < p.shared_probes; ++i) {
-          uint64_t cur = *(volatile uint64_t*)(sk + s);
-          if (cur == 0) {
-            cur = atomicCAS((unsigned long long*)(sk + s), 0ull, (unsigned long long)ek[j]);
-            if (cur == 0) cur = ek[j];
-          }
-          if (cur == ek[j]) {
-            unsigned long long* t = sa + (size_t)s * NA;
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-              if (umax_word<NA>(a)) {  // raise only when the row improves it
-                if (w[a] > *(volatile unsigned long long*)(t + a))
-                  atomicMax(t + a, (unsigned long long)w[a]);
-              } else {
-                sadd64(t + a, w[a]);
-              }
-            }
-            placed = true;
-            break;
-          }
-          s = (s + 1) & (p.smem_slots - 1);
-        }
-        if (placed) continue;
-      }
       need[j] = true;
     }
     // global table: first slot reads of every remaining row, then resolve
@@ -246,7 +214,7 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
     }
   }
 
-  // fold the thread-private words and the shared table into the global table
+  // fold the thread-private words into the global table
   if (PIN) {
     const int lane = tid & 31;
     for (int d = 0; d < PM; ++d) {
@@ -274,15 +242,105 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
     for (int a = 0; a < NA; ++a) w[a] = csum[tid * NA + a];
     global_update<NA>(p, pkd[tid], w);
   }
-  if (SMT) {
-    for (uint32_t s = tid; s < p.smem_slots; s += ST_BLOCK) {
-      const uint64_t k = sk[s];
-      if (k == 0) continue;
-      uint64_t w[NA];
+}
+
+// A row outside the fast path, out of line: INT64_MIN to the side accumulator,
+// any other key to the global table.
+template <int NA>
+__device__ __noinline__ void rare_row(const GbParams& p, uint64_t ek, uint64_t val) {
+  uint64_t w[NA];
+  words_of<NA>(val, w);
+  if (ek == 0) {
+    atomicAdd(&p.hdr->n_side, 1ull);
+    red_global<NA>(p.hdr->side_aggs, w);
+  } else {
+    global_update<NA>(p, ek, w);
+  }
+}
+
+// Rows into one shared-memory table per CTA (a plan with CTA-shared slots),
+// merged into the global table at the end; rows the table has no room for go
+// to the global table one by one.  Pinned and thread-private slots of the plan
+// are not used: on a hot key the table's adds serialise over a warp's lanes
+// (15 ns a warp at worst), less than a second lookup costs every row.
+constexpr int SG_U = 4;            // rows per thread per chunk
+constexpr uint32_t SG_MAX_BYTES = 200 * 1024;
+
+template <class KT, int NA>
+__global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbParams p) {
+  extern __shared__ __align__(16) uint8_t sm[];
+  SmTab<NA> t;
+  t.bind(sm, p.smem_slots);
+  t.clear();
+  const int tid = threadIdx.x, B = blockDim.x;
+  const KT* keys = (const KT*)p.col[p.key_col[0]];
+  const int64_t* vals = (const int64_t*)p.col[p.r_a];
+  const int64_t n = p.n_rows;
+  const int64_t CHUNK = (int64_t)B * SG_U, step = (int64_t)gridDim.x * CHUNK;
+  const bool vec = ((uintptr_t)keys % (2 * sizeof(KT)) == 0) && ((uintptr_t)vals % 16 == 0);
+  // rows base + j * 2 * B + 2 * tid + {0, 1}; the next chunk's loads go out
+  // before this chunk is worked on
+  auto load = [&](int64_t base, uint64_t(&ek)[SG_U], uint64_t(&val)[SG_U]) -> uint32_t {
+    uint32_t ok = 0;
+    if (vec && base + CHUNK <= n) {
 #pragma unroll
-      for (int a = 0; a < NA; ++a) w[a] = sa[(size_t)s * NA + a];
-      global_update<NA>(p, k, w);
+      for (int j = 0; j < SG_U / 2; ++j) {
+        const int64_t r = base + (int64_t)j * 2 * B + 2 * tid;
+        int64_t k0, k1;
+        KeyPair<KT>::split(__ldcs((const typename KeyPair<KT>::V*)(keys + r)), k0, k1);
+        const longlong2 vv = __ldcs((const longlong2*)(vals + r));
+        ek[2 * j] = (uint64_t)k0 ^ KEY_FLIP;
+        ek[2 * j + 1] = (uint64_t)k1 ^ KEY_FLIP;
+        val[2 * j] = (uint64_t)vv.x;
+        val[2 * j + 1] = (uint64_t)vv.y;
+      }
+      return (1u << SG_U) - 1;
     }
+#pragma unroll
+    for (int j = 0; j < SG_U; ++j) {
+      const int64_t r = base + (int64_t)(j / 2) * 2 * B + 2 * tid + (j & 1);
+      const bool in = r < n;
+      ek[j] = in ? (uint64_t)(int64_t)keys[r] ^ KEY_FLIP : 0;
+      val[j] = in ? (uint64_t)vals[r] : 0;
+      ok |= (in ? 1u : 0u) << j;
+    }
+    return ok;
+  };
+  uint64_t ek[SG_U], val[SG_U];
+  uint32_t ok = 0;
+  int64_t base = (int64_t)blockIdx.x * CHUNK;
+  if (base < n) ok = load(base, ek, val);
+  __syncthreads();
+  for (; base < n; base += step) {
+    uint64_t nek[SG_U], nval[SG_U];
+    uint32_t nok = 0;
+    if (base + step < n) nok = load(base + step, nek, nval);
+    uint32_t rare = 0, slot[SG_U];  // INT64_MIN rows, and those without a slot
+#pragma unroll
+    for (int j = 0; j < SG_U; ++j) rare |= (ek[j] == 0 ? 1u : 0u) << j;
+    rare &= ok;
+    rare |= t.find(ek, (int)p.shared_probes, slot);
+    if (rare) {
+#pragma unroll
+      for (int j = 0; j < SG_U; ++j)
+        if (rare >> j & 1) rare_row<NA>(p, ek[j], val[j]);
+    }
+    __syncwarp();
+    t.add(slot, val);
+#pragma unroll
+    for (int j = 0; j < SG_U; ++j) {
+      ek[j] = nek[j];
+      val[j] = nval[j];
+    }
+    ok = nok;
+  }
+  __syncthreads();
+  for (uint32_t s = tid; s < p.smem_slots; s += B) {
+    const uint64_t k = t.key_of(s);
+    if (k == 0) continue;
+    uint64_t w[NA];
+    t.words(s, w);
+    global_update<NA>(p, k, w);
   }
 }
 
@@ -611,29 +669,28 @@ rel_status ppass_dispatch(const GbParams& p, bool scatter, cudaStream_t st) {
   return scatter ? launch_ppass<KT, NA, false, true>(p, st) : launch_ppass<KT, NA, false, false>(p, st);
 }
 
-size_t stream_smem(int na, bool pin, bool smt, uint32_t smem_slots) {
+size_t stream_smem(int na, bool pin) {
   size_t b = 416 + 8 * ST_PIN_LIMIT * 4;
   if (pin) b += (size_t)8 * (na == 4 ? pin_max<4>() : pin_max<2>()) * na * ST_BLOCK;
-  if (smt) b += (size_t)8 * smem_slots * (1 + na);
   return b;
 }
 
-template <class KT, int NA, bool PIN, bool SMT>
-rel_status launch_stream(const GbParams& p, cudaStream_t st) {
-  auto kern = gb_stream_k<KT, NA, PIN, SMT>;
-  const size_t smem = stream_smem(NA, PIN, SMT, p.smem_slots);
+// One wave of resident CTAs, at most one per chunk.
+template <class K>
+rel_status launch_rows(K kern, int block, size_t smem, int64_t chunk, const GbParams& p,
+                       cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(stream)");
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, ST_BLOCK, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "occupancy(stream)");
   if (occ < 1) return relhost::set_error("group-by: stream kernel does not fit"), REL_E_UNSUPPORTED;
-  const int64_t chunks = (p.n_rows + (int64_t)ST_BLOCK * ST_U - 1) / ((int64_t)ST_BLOCK * ST_U);
+  const int64_t chunks = (p.n_rows + chunk - 1) / chunk;
   int64_t grid = (int64_t)relhost::device_sms() * occ;
   if (grid > chunks) grid = chunks;
   if (grid < 1) grid = 1;
   relhost::launch_begin(relhost::K_GB_STREAM, st);
-  kern<<<(int)grid, ST_BLOCK, smem, st>>>(p);
+  kern<<<(int)grid, block, smem, st>>>(p);
   relhost::launch_end(relhost::K_GB_STREAM, st);
   e = cudaGetLastError();
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(stream)");
@@ -641,12 +698,28 @@ rel_status launch_stream(const GbParams& p, cudaStream_t st) {
 
 template <class KT, int NA>
 rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
+  if (p.smem_slots) {
+    // 1024 resident threads per SM whatever the table's size; small inputs in
+    // small CTAs, so that more SMs take part
+    const int64_t small = (int64_t)relhost::device_sms() * 2048;
+    GbParams q = p;
+    // a plan's table is half full; where the rows pay for clearing and merging
+    // it, up to four times the slots keep more keys in their home bucket (1e8
+    // rows, 400 groups: 1024 slots 0.64 ms, 4096 slots 0.50 ms), as long as two
+    // CTAs fit -- and a table that would be nearly full is doubled once more
+    if (p.n_rows > 8 * small)
+      while (q.smem_slots < 4 * p.smem_slots && SmTab<NA>::bytes(2 * q.smem_slots) <= 110 * 1024)
+        q.smem_slots *= 2;
+    if (NA == 2 && q.smem_slots == SHARED_MAX_SLOTS && q.smem_slots == p.smem_slots)
+      q.smem_slots *= 2;
+    const size_t smem = SmTab<NA>::bytes(q.smem_slots);
+    const int block = smem > 110 * 1024 ? 1024 : smem > 54 * 1024 || p.n_rows > small ? 512 : 256;
+    return launch_rows(gb_smem_k<KT, NA>, block, smem, (int64_t)block * SG_U, q, st);
+  }
   const bool pin = p.tiny_frozen && p.tiny_slots;
-  const bool smt = p.smem_slots != 0;
-  if (pin && smt) return launch_stream<KT, NA, true, true>(p, st);
-  if (pin) return launch_stream<KT, NA, true, false>(p, st);
-  if (smt) return launch_stream<KT, NA, false, true>(p, st);
-  return launch_stream<KT, NA, false, false>(p, st);
+  const size_t smem = stream_smem(NA, pin);
+  if (pin) return launch_rows(gb_stream_k<KT, NA, true>, ST_BLOCK, smem, ST_BLOCK * ST_U, p, st);
+  return launch_rows(gb_stream_k<KT, NA, false>, ST_BLOCK, smem, ST_BLOCK * ST_U, p, st);
 }
 
 }  // namespace
@@ -655,15 +728,14 @@ bool gb_stream_eligible(const GbParams& p, int shape, int n_hot) {
   const bool kv = shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
                   shape == SHAPE_KV2_32;
   if (!kv) return false;
+  const int na = (shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32) ? 4 : 2;
+  // a CTA-shared table: gb_smem_k
+  if (p.smem_slots)
+    return (na == 4 ? SmTab<4>::bytes(p.smem_slots) : SmTab<2>::bytes(p.smem_slots)) <= SG_MAX_BYTES;
   // thread-private slots only when pinned (a first-come thread-private
   // table is the fused kernel's job)
-  const int na = (shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32) ? 4 : 2;
-  const bool pin = p.tiny_slots != 0;
   const int pmax = na == 4 ? pin_max<4>() : pin_max<2>();
-  if (pin && !(p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= pmax)) return false;
-  // a large shared table would leave too few resident threads for the
-  // global probes' latency: that case stays with the fused kernel
-  return stream_smem(na, pin, p.smem_slots != 0, p.smem_slots) <= 80 * 1024;
+  return !p.tiny_slots || (p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= pmax);
 }
 
 // Level 2 of the streaming scatter: every tile of PART_TILE level-1 records
