@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "batch.cuh"
+#include "smtab.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -29,19 +30,41 @@ namespace rel {
 
 namespace {
 
-constexpr uint32_t BATCH_SMEM_MULT = 0x9E3779B1u;
 constexpr int BATCH_SMEM_PROBES = 32;
 
+// Instance of a work item (start[i] <= item < start[i + 1]), found by a whole
+// warp: every round splits the range 32 ways, so 4096 instances take three
+// dependent loads instead of twelve.
 __device__ __forceinline__ int find_instance(const long long* start, int n, long long item) {
-  int lo = 0, hi = n;  // start[lo] <= item < start[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(start + mid) <= item)
-      lo = mid;
-    else
-      hi = mid;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, len = n;  // start[lo] <= item < start[lo + len]
+  while (len > 1) {
+    const int step = (len + 31) >> 5;
+    const int at = lo + lane * step;
+    const bool le = lane * step < len && __ldg(start + at) <= item;
+    const int k = 31 - __clz(__ballot_sync(0xffffffffu, le));  // lane 0 always votes
+    lo += k * step;
+    len = len - k * step < step ? len - k * step : step;
   }
   return lo;
+}
+
+// The next work item of a launch (warp 0): total items, the first `split` of
+// which belong to `first`, the rest to `second`; *inst < 0 when none is left.
+__device__ __forceinline__ void next_item(unsigned long long* ctr, long long total, long long split,
+                                          const long long* first, int n_first,
+                                          const long long* second, int n_second,
+                                          long long* item, int* inst) {
+  unsigned long long t = 0;
+  if ((threadIdx.x & 31) == 0) t = atomicAdd(ctr, 1ull);
+  const long long x = (long long)__shfl_sync(0xffffffffu, t, 0);
+  const int i = x >= total  ? -1
+                : x < split ? find_instance(first, n_first, x)
+                            : find_instance(second, n_second, x - split);
+  if ((threadIdx.x & 31) == 0) {
+    *item = x;
+    *inst = i;
+  }
 }
 
 __device__ __forceinline__ uint64_t encode_word(int op, int64_t v) {
@@ -53,17 +76,9 @@ __device__ __forceinline__ uint64_t encode_word(int op, int64_t v) {
 
 __device__ __forceinline__ void red_global(unsigned long long* w, int op, uint64_t x) {
   if (op == REL_MIN || op == REL_MAX)
-    atomicMax(w, (unsigned long long)x);
+    redg_max(w, x);
   else
-    atomicAdd(w, (unsigned long long)x);
-}
-
-__device__ __forceinline__ void red_shared(unsigned long long* w, int op, uint64_t x) {
-  if (op == REL_MIN || op == REL_MAX) {
-    if (x > *(volatile unsigned long long*)w) atomicMax(w, (unsigned long long)x);
-  } else {
-    sadd64(w, x);
-  }
+    redg_add(w, x);
 }
 
 // The encoded words of one row (or of a pre-aggregated slot) for aggregate a.
@@ -89,31 +104,56 @@ __device__ __forceinline__ void side_update(const BatchGb& g, BatchStatus* st, c
   red_words(g, st->side_aggs, x);
 }
 
-// One thread: insert-or-accumulate encoded words into the global table,
-// starting from slot s whose content cur was already loaded.
-__device__ __forceinline__ void global_resolve(const BatchGb& g, BatchStatus* st, uint64_t ek,
-                                               uint64_t s, uint64_t cur, const Words& x) {
+// Global tables are walked from the first slot of the key's home sector (four
+// keys, 32 bytes): one 256-bit load shows four slots for the price of one, so
+// at most half load 97 of 100 rows end at their first load.
+__device__ __forceinline__ uint64_t home_slot(const BatchGb& g, uint64_t ek) {
+  return slot_of(ek, g.log2_slots) & ~3ull;
+}
+__device__ __forceinline__ void ld_sector(const uint64_t* p, uint64_t (&k)[4]) {
+  asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(k[0]), "=l"(k[1]), "=l"(k[2]), "=l"(k[3])
+               : "l"(p)
+               : "memory");
+}
+
+// Slot of ek at or after slot s (the first of a sector), claiming the first
+// empty one; ~0 when the table overflowed.  Out of line: the rare path.
+__device__ __noinline__ uint64_t global_claim(const BatchGb& g, BatchStatus* st, uint64_t ek,
+                                              uint64_t s) {
   const uint64_t mask = (1ull << g.log2_slots) - 1;
-  for (uint32_t i = 0; i < g.max_probe; ++i) {
-    if (i) cur = ld_relaxed(g.tkeys + s);
-    if (cur == 0) {
-      cur = atomicCAS((unsigned long long*)(g.tkeys + s), 0ull, (unsigned long long)ek);
-      if (cur == 0) cur = ek;
+  for (uint32_t i = 0; i < g.max_probe; i += 4) {
+    uint64_t k[4];
+    ld_sector(g.tkeys + s, k);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (k[q] == 0) {
+        k[q] = atomicCAS((unsigned long long*)(g.tkeys + s + q), 0ull, (unsigned long long)ek);
+        if (k[q] == 0) k[q] = ek;
+      }
+      if (k[q] == ek) return s + q;
     }
-    if (cur == ek) {
-      red_words(g, g.taggs + s * (uint64_t)g.n_aggs, x);
-      return;
-    }
-    s = (s + 1) & mask;
-    if ((i & 31) == 31 && ld_relaxed_u32(&st->overflow)) return;  // already overflowed
+    s = (s + 4) & mask;
+    if ((i & 31) == 28 && ld_relaxed_u32(&st->overflow)) return ~0ull;  // already overflowed
   }
   atomicOr(&st->overflow, 1u);
+  return ~0ull;
 }
 
 __device__ __forceinline__ void global_update(const BatchGb& g, BatchStatus* st, uint64_t ek,
                                               const Words& x) {
-  const uint64_t s = slot_of(ek, g.log2_slots);
-  global_resolve(g, st, ek, s, ld_relaxed(g.tkeys + s), x);
+  const uint64_t s = global_claim(g, st, ek, home_slot(g, ek));
+  if (s != ~0ull) red_words(g, g.taggs + s * (uint64_t)g.n_aggs, x);
+}
+
+// A row outside the fast paths, out of line: INT64_MIN to the side
+// accumulator, any other key to the global table.
+__device__ __noinline__ void rare_row(const BatchGb& g, BatchStatus* st, uint64_t ek, uint64_t v) {
+  const Words x = row_words(g, (int64_t)v);
+  if (ek == 0)
+    side_update(g, st, x);
+  else
+    global_update(g, st, ek, x);
 }
 
 // W threads probe together: each reads one slot of a W-slot window; a key
@@ -136,7 +176,7 @@ __device__ __noinline__ void global_update_coop(const BatchGb& g, BatchStatus* s
       if (rank == 0) side_update(g, st, x);
       continue;
     }
-    const uint64_t base = slot_of(k, g.log2_slots);
+    const uint64_t base = home_slot(g, k);
     bool done = false;
     for (uint32_t i = 0; i < g.max_probe && !done; i += W) {
       if ((i & 31) == 32 - W && tile.any(ld_relaxed_u32(&st->overflow) != 0)) {
@@ -171,148 +211,257 @@ __device__ __noinline__ void global_update_coop(const BatchGb& g, BatchStatus* s
   }
 }
 
-// One tile of B x ITEMS rows starting at row r0: each row goes to the
-// shared-memory table (when the instance has one) or the global table.
-template <int ITEMS, int W>
-__device__ __forceinline__ void gb_rows(const BatchGb& g, BatchStatus* st, long long r0,
-                                        uint64_t* smk, unsigned long long* sma) {
+// Rows base + j / 2 * 2 * B + 2 * tid + {0, 1} (j < U) below end; ek = 0 where
+// there is none.  vec: both columns allow two rows per load.
+template <class KT, int U>
+__device__ __forceinline__ uint32_t load_rows(const BatchGb& g, bool vec, long long base,
+                                              long long end, uint64_t (&ek)[U], uint64_t (&v)[U]) {
+  const KT* keys = (const KT*)g.keys;
   const int B = blockDim.x;
-  uint64_t ek[ITEMS];
-  int64_t vv[ITEMS];
-  bool ok[ITEMS];
+  if (vec && base + (long long)B * U <= end) {
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const long long r = r0 + (long long)j * B + threadIdx.x;
-    ok[j] = r < g.n_rows;
-    int64_t k = 0, v = 0;
-    if (ok[j]) {
-      k = g.key_type == REL_I32 ? (int64_t)__ldcs((const int*)g.keys + r)
-                                : (int64_t)__ldcs((const long long*)g.keys + r);
-      if (g.vals) v = (int64_t)__ldcs((const long long*)g.vals + r);
-    }
-    ek[j] = (uint64_t)k ^ KEY_FLIP;
-    vv[j] = v;
-  }
-  if (g.smem_slots) {
-    const uint32_t S = (uint32_t)g.smem_slots, A = (uint32_t)g.n_aggs;
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      if (!ok[j]) continue;
-      const Words x = row_words(g, vv[j]);
-      if (ek[j] == 0) {
-        side_update(g, st, x);
-        continue;
+    for (int j = 0; j < U; j += 2) {
+      const long long r = base + (long long)j * B + 2 * threadIdx.x;
+      if constexpr (sizeof(KT) == 8) {
+        const longlong2 k = __ldcs((const longlong2*)(keys + r));
+        ek[j] = (uint64_t)k.x ^ KEY_FLIP;
+        ek[j + 1] = (uint64_t)k.y ^ KEY_FLIP;
+      } else {
+        const int2 k = __ldcs((const int2*)(keys + r));
+        ek[j] = (uint64_t)(int64_t)k.x ^ KEY_FLIP;
+        ek[j + 1] = (uint64_t)(int64_t)k.y ^ KEY_FLIP;
       }
-      uint32_t s = small_slot_of(ek[j], S - 1, BATCH_SMEM_MULT);
-      bool placed = false;
-      for (int i = 0; i < BATCH_SMEM_PROBES; ++i) {
-        uint64_t cur = *(volatile uint64_t*)(smk + s);
-        if (cur == 0) {
-          cur = atomicCAS((unsigned long long*)(smk + s), 0ull, (unsigned long long)ek[j]);
-          if (cur == 0) cur = ek[j];
-        }
-        if (cur == ek[j]) {
-#pragma unroll
-          for (int a = 0; a < BATCH_MAX_AGGS; ++a)
-            if (a < (int)A) red_shared(sma + (size_t)s * A + a, g.ops[a], x.w[a]);
-          placed = true;
-          break;
-        }
-        s = (s + 1) & (S - 1);
-      }
-      if (!placed) global_update(g, st, ek[j], x);
+      const longlong2 x = __ldcs((const longlong2*)(g.vals + r));
+      v[j] = (uint64_t)x.x;
+      v[j + 1] = (uint64_t)x.y;
     }
-    return;
+    return (1u << U) - 1;
   }
-  if (W == 1) {
-    // every row's first slot is read before any row is resolved: ITEMS
-    // independent L2 round trips in flight per thread instead of one
-    uint64_t gs[ITEMS], gk[ITEMS];
+  uint32_t ok = 0;
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      gs[j] = slot_of(ek[j], g.log2_slots);
-      gk[j] = (ok[j] && ek[j] != 0) ? ld_relaxed(g.tkeys + gs[j]) : 0;
+  for (int j = 0; j < U; ++j) {
+    const long long r = base + (long long)(j / 2) * 2 * B + 2 * threadIdx.x + (j & 1);
+    const bool in = r < end;
+    ek[j] = in ? (uint64_t)(int64_t)__ldcs(keys + r) ^ KEY_FLIP : 0;
+    v[j] = in && g.vals ? (uint64_t)__ldcs((const long long*)g.vals + r) : 0;
+    ok |= (in ? 1u : 0u) << j;
+  }
+  return ok;
+}
+
+// Rows into the CTA's shared-memory table (smtab.cuh), cleared before and
+// merged into the instance's global table after: one update per distinct key
+// of the work item.
+template <class KT, int NA>
+__device__ __noinline__ void shared_rows(const BatchGb& g, BatchStatus* st, long long r0,
+                                            long long r1, uint8_t* sm) {
+  constexpr int U = NA == 4 ? 2 : 4;  // rows per thread in flight (registers)
+  SmTab<NA> t;
+  t.bind(sm, (uint32_t)g.smem_slots);
+  t.clear();
+  const bool vec = g.vals && (uintptr_t)g.keys % (2 * sizeof(KT)) == 0 && (uintptr_t)g.vals % 16 == 0;
+  const long long step = (long long)blockDim.x * U;
+  uint64_t ek[U], v[U];
+  uint32_t ok = load_rows<KT, U>(g, vec, r0, r1, ek, v);
+  __syncthreads();
+  for (; r0 < r1; r0 += step) {
+    uint64_t nek[U], nv[U];
+    const uint32_t nok = load_rows<KT, U>(g, vec, r0 + step, r1, nek, nv);
+    uint32_t rare = 0, slot[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) rare |= (ek[j] == 0 ? 1u : 0u) << j;
+    rare &= ok;
+    rare |= t.find(ek, BATCH_SMEM_PROBES, slot);
+    if (rare) {
+#pragma unroll
+      for (int j = 0; j < U; ++j)
+        if (rare >> j & 1) rare_row(g, st, ek[j], v[j]);
     }
+    __syncwarp();
+    t.add(slot, v);
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      if (!ok[j]) continue;
-      const Words x = row_words(g, vv[j]);
-      if (ek[j] == 0)
-        side_update(g, st, x);
-      else
-        global_resolve(g, st, ek[j], gs[j], gk[j], x);
+    for (int j = 0; j < U; ++j) {
+      ek[j] = nek[j];
+      v[j] = nv[j];
     }
-  } else {
+    ok = nok;
+  }
+  __syncthreads();
+  for (uint32_t s = threadIdx.x; s < (uint32_t)g.smem_slots; s += blockDim.x) {
+    const uint64_t k = t.key_of(s);
+    if (k == 0) continue;
+    uint64_t w[NA];
+    t.words(s, w);
+    Words x;
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) global_update_coop<W>(g, st, ek[j], vv[j], ok[j]);
+    for (int a = 0; a < BATCH_MAX_AGGS; ++a) {
+      x.w[a] = 0;
+      if (a < g.n_aggs) {
+        const int op = g.ops[a];
+        x.w[a] = op == REL_SUM ? w[0] : w[1];
+        if constexpr (NA == 4) x.w[a] = op == REL_MIN ? w[2] : op == REL_MAX ? w[3] : x.w[a];
+      }
+    }
+    global_update(g, st, k, x);
+  }
+  __syncthreads();
+}
+
+// Rows straight into the instance's global table (W = 1): two home sectors in
+// flight per thread, then both rows' reductions.  The few rows that leave
+// their home sector are finished in a loop of their own, inline: a call there
+// would store its caller's registers to local memory for every warp (7 rows in
+// 10 have such a lane), which writes through to L2 beside the reductions.
+template <class KT>
+__device__ __noinline__ void global_rows(const BatchGb& g, BatchStatus* st, long long r0,
+                                         long long r1) {
+  constexpr int U = 2;
+  const bool vec = g.vals && (uintptr_t)g.keys % (2 * sizeof(KT)) == 0 && (uintptr_t)g.vals % 16 == 0;
+  const long long step = (long long)blockDim.x * U;
+  uint64_t* const tk = g.tkeys;
+  unsigned long long* const ta = g.taggs;
+  const uint64_t mask = (1ull << g.log2_slots) - 1;
+  for (; r0 < r1; r0 += step) {
+    uint64_t ek[U], v[U], s[U];
+    const uint32_t ok = load_rows<KT, U>(g, vec, r0, r1, ek, v);
+    uint32_t miss = 0, put = ok;
+    {
+      uint64_t k[U][4];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        s[j] = home_slot(g, ek[j]);
+        ld_sector(tk + s[j], k[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const uint64_t e = ek[j];
+        const uint32_t at = k[j][0] == e ? 0 : k[j][1] == e ? 1 : k[j][2] == e ? 2 : k[j][3] == e ? 3 : 4;
+        if (at == 4) {
+          miss |= 1u << j;
+          if (k[j][3] != 0) s[j] = (s[j] + 4) & mask;  // the home sector is full
+        } else {
+          s[j] += at;
+        }
+        if (e == 0) {  // no row, or INT64_MIN
+          if (ok >> j & 1) rare_row(g, st, 0, v[j]);
+          put &= ~(1u << j);
+        }
+      }
+    }
+    miss &= put;
+    for (uint32_t i = 0; miss; i += 4) {
+      const bool second = !(miss & 1);
+      const uint64_t e = second ? ek[1] : ek[0];
+      uint64_t w = second ? s[1] : s[0], k[4];
+      ld_sector(tk + w, k);
+      uint32_t at = k[0] == e ? 0 : k[1] == e ? 1 : k[2] == e ? 2 : k[3] == e ? 3 : 4;
+      if (at == 4 && k[3] == 0) {  // room as loaded: claim the first empty slot
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (at != 4 || k[q] != 0) continue;
+          const uint64_t old = atomicCAS((unsigned long long*)(tk + w + q), 0ull, (unsigned long long)e);
+          if (old == 0 || old == e) at = q;
+        }
+      }
+      bool done = at != 4;
+      w = done ? w + at : (w + 4) & mask;
+      if (!done && ((i & 31) == 28 && ld_relaxed_u32(&st->overflow))) {  // already overflowed
+        done = true;
+        put &= ~(miss & (0u - miss));
+      } else if (!done && i >= 2 * g.max_probe) {
+        atomicOr(&st->overflow, 1u);
+        done = true;
+        put &= ~(miss & (0u - miss));
+      }
+      if (second) s[1] = w; else s[0] = w;
+      if (done) miss &= miss - 1;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (put >> j & 1) red_words(g, ta + s[j] * (uint64_t)g.n_aggs, row_words(g, (int64_t)v[j]));
   }
 }
 
-// Work item t of a group-by: g.span consecutive tiles.  With a shared-memory
-// table the item pre-aggregates all its rows there (cleared once, flushed to
-// the global table once, one update per distinct key).
+// Work item t of a group-by: g.span consecutive tiles of B x ITEMS rows.
 template <int ITEMS, int W>
 __device__ __forceinline__ void gb_tile(const BatchGb& g, BatchStatus* st, long long t,
-                                        uint64_t* smk, unsigned long long* sma) {
+                                        uint8_t* sm) {
   const int B = blockDim.x;
-  const long long T = (long long)B * ITEMS;
-  const long long first = t * (long long)g.span;
-  const long long last = (g.n_rows + T - 1) / T < first + g.span ? (g.n_rows + T - 1) / T
-                                                                 : first + g.span;
-  const uint32_t S = (uint32_t)g.smem_slots, A = (uint32_t)g.n_aggs;
-  if (S) {
-    for (uint32_t i = threadIdx.x; i < S * (1 + A); i += B) smk[i] = 0;
-    __syncthreads();
-  }
-  for (long long k = first; k < last; ++k) gb_rows<ITEMS, W>(g, st, k * T, smk, sma);
-  if (S) {
-    __syncthreads();
-    for (uint32_t s = threadIdx.x; s < S; s += B) {
-      const uint64_t k = smk[s];
-      if (k == 0) continue;
-      Words x;
-#pragma unroll
-      for (int a = 0; a < BATCH_MAX_AGGS; ++a) x.w[a] = a < (int)A ? sma[(size_t)s * A + a] : 0;
-      global_update(g, st, k, x);
+  const long long rows = (long long)B * ITEMS * g.span;
+  const long long r0 = t * rows, r1 = r0 + rows < g.n_rows ? r0 + rows : g.n_rows;
+  const bool k32 = g.key_type == REL_I32;
+  if (g.smem_slots) {
+    bool minmax = false;
+    for (int a = 0; a < g.n_aggs; ++a) minmax |= g.ops[a] == REL_MIN || g.ops[a] == REL_MAX;
+    if (minmax)
+      k32 ? shared_rows<int, 4>(g, st, r0, r1, sm) : shared_rows<long long, 4>(g, st, r0, r1, sm);
+    else
+      k32 ? shared_rows<int, 2>(g, st, r0, r1, sm) : shared_rows<long long, 2>(g, st, r0, r1, sm);
+  } else if (W == 1) {
+    k32 ? global_rows<int>(g, st, r0, r1) : global_rows<long long>(g, st, r0, r1);
+  } else {
+    for (long long r = r0; r < r1; r += B) {
+      const long long i = r + threadIdx.x;
+      const bool in = i < r1;
+      int64_t k = 0, v = 0;
+      if (in) {
+        k = k32 ? (int64_t)__ldcs((const int*)g.keys + i) : (int64_t)__ldcs((const long long*)g.keys + i);
+        if (g.vals) v = (int64_t)__ldcs((const long long*)g.vals + i);
+      }
+      global_update_coop<W>(g, st, (uint64_t)k ^ KEY_FLIP, v, in);
     }
-    __syncthreads();
   }
 }
 
+// Build rows into their partition's table: every build row claims the first
+// empty slot from its home sector on.  The table is at most half full, so the
+// home sector's first slot is tried without a look, BUILD_U rows at a time.
 template <int ITEMS>
 __device__ __forceinline__ void build_tile(const BatchJoin& J, BatchStatus* st, long long t) {
+  constexpr int BUILD_U = 4;
   const int B = blockDim.x;
-  const long long r0 = t * (long long)B * ITEMS;
   const uint64_t mask = (1ull << J.log2_slots) - 1;
+  for (int j0 = 0; j0 < ITEMS; j0 += BUILD_U) {
+    const long long r0 = t * (long long)B * ITEMS + (long long)j0 * B + threadIdx.x;
+    uint64_t ek[BUILD_U], s[BUILD_U];
+    JoinVal v[BUILD_U];
+    unsigned long long got[BUILD_U];
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const long long r = r0 + (long long)j * B + threadIdx.x;
-    if (r >= J.n_build) continue;
-    const uint64_t ek = (uint64_t)__ldg((const long long*)J.bkeys + r) ^ KEY_FLIP;
-    const JoinVal v{__ldg((const long long*)J.bpay + r), (int32_t)r, 0};
-    if (ek == 0) {
-      const unsigned long long pos = atomicAdd(&st->n_side, 1ull);
-      J.side[pos] = v;
-      continue;
+    for (int j = 0; j < BUILD_U; ++j) {
+      const long long r = r0 + (long long)j * B;
+      const bool in = r < J.n_build;
+      ek[j] = in ? (uint64_t)__ldcs((const long long*)J.bkeys + r) ^ KEY_FLIP : 0;
+      v[j] = JoinVal{in ? __ldcs((const long long*)J.bpay + r) : 0, (int32_t)r, 0};
+      if (in && ek[j] == 0) J.side[atomicAdd(&st->n_side, 1ull)] = v[j];
     }
-    uint64_t s = slot_of(ek, J.log2_slots);
-    bool placed = false;
-    for (uint32_t i = 0; i < J.max_probe; ++i) {
-      if (ld_relaxed(J.tkeys + s) == 0 &&
-          atomicCAS((unsigned long long*)(J.tkeys + s), 0ull, (unsigned long long)ek) == 0) {
-        J.tvals[s] = v;
-        placed = true;
-        break;
+#pragma unroll
+    for (int j = 0; j < BUILD_U; ++j) {
+      s[j] = slot_of(ek[j], J.log2_slots) & ~3ull;
+      got[j] = 1;
+      if (ek[j] != 0)
+        got[j] = atomicCAS((unsigned long long*)(J.tkeys + s[j]), 0ull, (unsigned long long)ek[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < BUILD_U; ++j) {
+      if (ek[j] == 0) continue;
+      for (uint32_t i = 0; got[j] != 0 && i < J.max_probe; ++i) {
+        s[j] = (s[j] + 1) & mask;
+        got[j] = ld_relaxed(J.tkeys + s[j]);
+        if (got[j] == 0)
+          got[j] = atomicCAS((unsigned long long*)(J.tkeys + s[j]), 0ull, (unsigned long long)ek[j]);
       }
-      s = (s + 1) & mask;
+      if (got[j] == 0)
+        J.tvals[s[j]] = v[j];
+      else
+        atomicOr(&st->overflow, 1u);
     }
-    if (!placed) atomicOr(&st->overflow, 1u);
   }
 }
 
 // Persistent launch A: join builds, then group-by tiles, from one counter.
 template <int ITEMS, int W>
-__global__ void __launch_bounds__(512) batch_a(const __grid_constant__ BatchArgs a) {
+__global__ void __launch_bounds__(512, 2) batch_a(const __grid_constant__ BatchArgs a) {
   extern __shared__ __align__(16) uint8_t bsm[];
   __shared__ long long s_item;
   __shared__ int s_inst;
@@ -320,19 +469,13 @@ __global__ void __launch_bounds__(512) batch_a(const __grid_constant__ BatchArgs
     BatchGb g;
     BatchJoin j;
   } s_desc;
-  uint64_t* smk = (uint64_t*)bsm;
   const long long n_build = a.n_j ? a.jb_tiles[a.n_j] : 0;
   const long long total = n_build + (a.n_g ? a.gb_tiles[a.n_g] : 0);
   for (;;) {
-    // one thread takes the next tile and finds its instance; the CTA copies
-    // that instance's descriptor into shared memory
-    if (threadIdx.x == 0) {
-      const long long item = (long long)atomicAdd(a.ctr, 1ull);
-      s_item = item;
-      s_inst = item >= total  ? -1
-               : item < n_build ? find_instance(a.jb_tiles, a.n_j, item)
-                                : find_instance(a.gb_tiles, a.n_g, item - n_build);
-    }
+    // warp 0 takes the next item and finds its instance; the CTA copies that
+    // instance's descriptor into shared memory
+    if (threadIdx.x < 32)
+      next_item(a.ctr, total, n_build, a.jb_tiles, a.n_j, a.gb_tiles, a.n_g, &s_item, &s_inst);
     __syncthreads();
     const long long item = s_item;
     const int i = s_inst;
@@ -347,9 +490,7 @@ __global__ void __launch_bounds__(512) batch_a(const __grid_constant__ BatchArgs
     if (is_build) {
       build_tile<ITEMS>(s_desc.j, a.jst + i, item - a.jb_tiles[i]);
     } else {
-      const BatchGb& g = s_desc.g;
-      unsigned long long* sma = (unsigned long long*)(smk + g.smem_slots);
-      gb_tile<ITEMS, W>(g, a.gst + i, item - n_build - a.gb_tiles[i], smk, sma);
+      gb_tile<ITEMS, W>(s_desc.g, a.gst + i, item - n_build - a.gb_tiles[i], bsm);
     }
     __syncthreads();
   }
@@ -397,63 +538,128 @@ __device__ __forceinline__ void compact_tile(const BatchGb& g, BatchStatus* st, 
   }
 }
 
-template <int ITEMS>
-__device__ __forceinline__ void probe_tile(const BatchJoin& J, BatchStatus* st, long long t) {
+// Matches of key e in the sector at slot s: bit q for slot s + q.  *last: an
+// empty slot ends the key's sequence (slots fill in order).
+__device__ __forceinline__ uint32_t match_sector(const uint64_t* tk, uint64_t s, uint64_t e,
+                                                 bool* last) {
+  uint64_t k[4];
+  asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(k[0]), "=l"(k[1]), "=l"(k[2]), "=l"(k[3])
+               : "l"(tk + s));
+  *last = k[3] == 0;
+  return (k[0] == e ? 1u : 0u) | (k[1] == e ? 2u : 0u) | (k[2] == e ? 4u : 0u) | (k[3] == e ? 8u : 0u);
+}
+
+// Probe rows [r0, r1): PROBE_U rows per thread have their home sectors and
+// first matches in flight together, and a warp's first matches take one output
+// claim; a row's further matches (build keys that repeat), sequences that go on
+// past the home sector and INT64_MIN rows are finished in a slower loop.
+__device__ __forceinline__ void probe_rows(const BatchJoin& J, BatchStatus* st, long long r0,
+                                           long long r1) {
+  constexpr int PROBE_U = 4;
   const int B = blockDim.x;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const uint64_t mask = (1ull << J.log2_slots) - 1;
-  const unsigned long long n_side = st->n_side;
-  const long long r0 = t * (long long)B * ITEMS;
-  for (int j = 0; j < ITEMS; ++j) {
-    const long long r = r0 + (long long)j * B + threadIdx.x;
-    const bool valid = r < J.n_probe;
-    const uint64_t ek = valid ? (uint64_t)__ldg((const long long*)J.pkeys + r) ^ KEY_FLIP : 0;
-    const bool side = valid && ek == 0;
-    uint64_t s = side ? 0 : slot_of(ek, J.log2_slots);
-    uint32_t steps = 0;
-    bool active = valid;
-    while (__any_sync(0xffffffffu, active)) {
-      bool hit = false;
-      JoinVal v{0, 0, 0};
-      if (active) {
-        // next match of this row's probe sequence
-        if (side) {
-          if (s < n_side) {
-            v = J.side[s++];
-            hit = true;
+  const unsigned long long n_side = st->n_side, cap = (unsigned long long)J.capacity;
+  for (; r0 < r1; r0 += (long long)B * PROBE_U) {
+    uint64_t ek[PROBE_U], s[PROBE_U];
+    uint32_t m[PROBE_U], more = 0, side = 0;
+#pragma unroll
+    for (int j = 0; j < PROBE_U; ++j) {
+      const long long r = r0 + (long long)j * B + threadIdx.x;
+      ek[j] = r < r1 ? (uint64_t)__ldcs((const long long*)J.pkeys + r) ^ KEY_FLIP : 0;
+      side |= (r < r1 && ek[j] == 0 ? 1u : 0u) << j;
+    }
+#pragma unroll
+    for (int j = 0; j < PROBE_U; ++j) {
+      s[j] = slot_of(ek[j], J.log2_slots) & ~3ull;
+      m[j] = 0;
+      bool last = true;
+      if (ek[j] != 0) m[j] = match_sector(J.tkeys, s[j], ek[j], &last);
+      more |= (last ? 0u : 1u) << j;
+    }
+    JoinVal v[PROBE_U];
+    uint32_t total = 0;
+#pragma unroll
+    for (int j = 0; j < PROBE_U; ++j) {
+      const unsigned h = __ballot_sync(0xffffffffu, m[j] != 0);
+      total += __popc(h);
+      if (m[j]) v[j] = J.tvals[s[j] + __ffs(m[j]) - 1];
+    }
+    if (total) {
+      unsigned long long wb = 0;
+      if (lane == 0) wb = atomicAdd(&st->n_out, (unsigned long long)total);
+      wb = __shfl_sync(0xffffffffu, wb, 0);
+#pragma unroll
+      for (int j = 0; j < PROBE_U; ++j) {
+        const unsigned h = __ballot_sync(0xffffffffu, m[j] != 0);
+        if (m[j]) {
+          const unsigned long long pos = wb + __popc(h & lt);
+          if (pos < cap) {
+            __stcs(J.o_pi + pos, (int32_t)(r0 + (long long)j * B + threadIdx.x));
+            __stcs(J.o_bi + pos, v[j].bidx);
+            __stcs((long long*)J.o_pay + pos, (long long)v[j].payload);
           }
-        } else {
-          while (steps < J.max_probe) {
-            const uint64_t k = J.tkeys[s];
-            if (k == 0) break;
-            const uint64_t cur = s;
-            s = (s + 1) & mask;
-            ++steps;
-            if (k == ek) {
-              v = J.tvals[cur];
+          m[j] &= m[j] - 1;
+        }
+        wb += __popc(h);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < PROBE_U; ++j) {
+      const bool sd = side >> j & 1;
+      bool go = sd || m[j] != 0 || (more >> j & 1);
+      uint64_t w = sd ? 0 : s[j];
+      uint32_t mm = m[j], steps = 0;
+      bool last = !(more >> j & 1);
+      while (__any_sync(0xffffffffu, go)) {
+        bool hit = false;
+        JoinVal x{0, 0, 0};
+        if (go) {
+          if (sd) {
+            if (w < n_side) {
+              x = J.side[w++];
               hit = true;
-              break;
+            }
+          } else {
+            while (mm == 0 && !last && steps < J.max_probe) {
+              w = (w + 4) & mask;
+              steps += 4;
+              mm = match_sector(J.tkeys, w, ek[j], &last);
+            }
+            if (mm) {
+              x = J.tvals[w + __ffs(mm) - 1];
+              mm &= mm - 1;
+              hit = true;
             }
           }
+          go = hit;
         }
-        active = hit;
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, hit);
-      if (!m) continue;
-      unsigned long long wb = 0;
-      if (lane == 0) wb = atomicAdd(&st->n_out, (unsigned long long)__popc(m));
-      wb = __shfl_sync(0xffffffffu, wb, 0);
-      if (hit) {
-        const unsigned long long pos = wb + __popc(m & lt);
-        if (pos < (unsigned long long)J.capacity) {
-          J.o_pi[pos] = (int32_t)r;
-          J.o_bi[pos] = v.bidx;
-          J.o_pay[pos] = v.payload;
+        const unsigned h = __ballot_sync(0xffffffffu, hit);
+        if (!h) continue;
+        unsigned long long wb = 0;
+        if (lane == 0) wb = atomicAdd(&st->n_out, (unsigned long long)__popc(h));
+        wb = __shfl_sync(0xffffffffu, wb, 0);
+        if (hit) {
+          const unsigned long long pos = wb + __popc(h & lt);
+          if (pos < cap) {
+            J.o_pi[pos] = (int32_t)(r0 + (long long)j * B + threadIdx.x);
+            J.o_bi[pos] = x.bidx;
+            J.o_pay[pos] = x.payload;
+          }
         }
       }
     }
   }
+}
+
+// Probe work item t of a join: J.span tiles.
+template <int ITEMS>
+__device__ __forceinline__ void probe_tile(const BatchJoin& J, BatchStatus* st, long long t) {
+  const long long rows = (long long)blockDim.x * ITEMS * J.span;
+  const long long r0 = t * rows;
+  probe_rows(J, st, r0, r0 + rows < J.n_probe ? r0 + rows : J.n_probe);
 }
 
 // Persistent launch B: join probes, then group-by compaction.
@@ -468,13 +674,8 @@ __global__ void __launch_bounds__(512) batch_b(const __grid_constant__ BatchArgs
   const long long n_probe = a.n_j ? a.jp_tiles[a.n_j] : 0;
   const long long total = n_probe + (a.n_g ? a.gc_tiles[a.n_g] : 0);
   for (;;) {
-    if (threadIdx.x == 0) {
-      const long long item = (long long)atomicAdd(a.ctr + 1, 1ull);
-      s_item = item;
-      s_inst = item >= total  ? -1
-               : item < n_probe ? find_instance(a.jp_tiles, a.n_j, item)
-                                : find_instance(a.gc_tiles, a.n_g, item - n_probe);
-    }
+    if (threadIdx.x < 32)
+      next_item(a.ctr + 1, total, n_probe, a.jp_tiles, a.n_j, a.gc_tiles, a.n_g, &s_item, &s_inst);
     __syncthreads();
     const long long item = s_item;
     const int i = s_inst;
@@ -511,7 +712,10 @@ rel_status launch_pair(const BatchArgs& a, int block, int smem, int grid_a, int 
 
 template <int ITEMS, int W>
 rel_status occ_pair(int block, int smem, int* pa, int* pb) {
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pa, batch_a<ITEMS, W>, block, smem);
+  cudaError_t e = cudaFuncSetAttribute(batch_a<ITEMS, W>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(batch)");
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pa, batch_a<ITEMS, W>, block, smem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pb, batch_b<ITEMS>, block, 0);
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "occupancy(batch)");
@@ -548,6 +752,13 @@ rel_status batch_launch(const BatchArgs& a, int block, int items, int width, int
     return launch_pair<decltype(I)::value, decltype(W)::value>(a, block, smem_bytes, grid_a,
                                                                grid_b, st);
   });
+}
+
+size_t batch_smem_bytes(const BatchGb& g) {
+  if (!g.smem_slots) return 0;
+  bool minmax = false;
+  for (int a = 0; a < g.n_aggs; ++a) minmax |= g.ops[a] == REL_MIN || g.ops[a] == REL_MAX;
+  return minmax ? SmTab<4>::bytes((uint32_t)g.smem_slots) : SmTab<2>::bytes((uint32_t)g.smem_slots);
 }
 
 rel_status batch_occupancy(int block, int items, int width, int smem_bytes, int* per_sm_a,

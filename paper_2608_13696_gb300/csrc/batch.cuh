@@ -14,6 +14,8 @@ constexpr int BATCH_MAX_SMEM_SLOTS = 4096;
 // descriptor copy, clearing and flushing a shared-memory table) are paid once
 // per ~64K rows rather than once per tile.
 constexpr int BATCH_GB_SPAN = 32;
+// ... and of one probe work item.
+constexpr int BATCH_JOIN_SPAN = 8;
 
 // One group-by instance as the kernels see it.
 struct alignas(16) BatchGb {
@@ -50,6 +52,8 @@ struct alignas(16) BatchJoin {
   int64_t capacity;
   int32_t log2_slots;
   uint32_t max_probe;
+  int32_t span;  // tiles of blockDim x ITEMS rows per probe work item
+  int32_t pad;
 };
 
 // Per-instance results, zeroed before every run.
@@ -79,6 +83,8 @@ struct BatchArgs {
 // the caller.
 rel_status batch_launch(const BatchArgs& a, int block, int items, int width, int smem_bytes,
                         int grid_a, int grid_b, cudaStream_t st);
+// Shared memory of a group-by instance's pre-aggregation table.
+size_t batch_smem_bytes(const BatchGb& g);
 rel_status batch_occupancy(int block, int items, int width, int smem_bytes, int* per_sm_a,
                            int* per_sm_b);
 
