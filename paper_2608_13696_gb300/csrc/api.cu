@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "distinct.cuh"
+#include "gen.cuh"
 #include "groupby.cuh"
 #include "join.cuh"
 #include "mlp.cuh"
@@ -393,7 +394,7 @@ rel_status run_main(GbParams& p, int shape, int mode, cudaStream_t st) {
       p.tiny_probes = 0;
     } else if (p.smem_slots > 16) {
       p.smem_slots >>= 1;
-    } else if (p.smem_slots && mode != MODE_KEYSET) {
+    } else if (p.smem_slots) {
       p.smem_slots = 0;
     } else {
       set_error("group-by: rows too wide to stage");
@@ -989,14 +990,6 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
       GbParams kp;
       const int ident[REL_MAX_AGGS] = {0, 1, 2, 3, 4, 5, 6, 7};
       fill_params(&kd, ident, kp);
-      // one int64 key and no filter: the specialised key/value reader, with
-      // the key column standing in as the (unused) value column
-      int kshape = SHAPE_GENERIC;
-      if (m.shape != SHAPE_GENERIC && kd.n_keys == 1 && kd.n_preds == 0 &&
-          kd.cols[keys[0]].type == REL_I64) {
-        kshape = SHAPE_KVRT64;
-        kp.r_a = keys[0];
-      }
       kp.hdr = (WsHeader*)ws;
       kp.tkeys = (uint64_t*)((uint8_t*)ws + HEADER_BYTES);
       const int32_t kt = kd.cols[keys[0]].type;
@@ -1013,11 +1006,9 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
         for (;;) {
           kp.log2_slots = log2_pow2(try_slots);
           kp.max_probe = (uint32_t)(try_slots < 4096 ? try_slots : 4096);
-          kp.smem_slots = 2048;
-          kp.shared_probes = 4;
           cudaError_t e = cudaMemsetAsync(ws, 0, HEADER_BYTES + 8ull * try_slots, st);
           if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemsetAsync");
-          if ((r = run_main(kp, kshape, MODE_KEYSET, st))) return r;
+          if ((r = gb_launch_gen_set(kp, st))) return r;
           HostHeader h;
           if ((r = read_header(ws, &h, st))) return r;
           if (h.timeout) return set_error("plan: a device wait timed out"), REL_E_TIMEOUT;
@@ -1536,9 +1527,11 @@ rel_status rel_groupby_agg(const rel_groupby_desc* d, const rel_plan* plan, void
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemsetAsync");
   if (plan->variant == REL_VAR_PARTITIONED && part_shape(m.shape)) {
     if ((r = run_partitioned(p, plan, m.shape, o, ws, st))) return r;
-  } else if (!(plan->flags & REL_PLAN_GENERIC) && !plan->tile_rows &&
-             gb_stream_eligible(p, m.shape, plan->n_hot)) {
+  } else if (!plan->tile_rows && gb_stream_shape(m.shape)) {
     if ((r = gb_launch_stream(p, m.shape, st))) return r;
+  } else if (!plan->tile_rows && (m.shape == SHAPE_GENERIC || m.shape == SHAPE_KVRT64 ||
+                                  m.shape == SHAPE_KVRT32)) {
+    if ((r = gb_launch_gen(p, plan->est_groups, st))) return r;
   } else {
     const int mode = p.tiny_ns ? MODE_TINY : MODE_LAYERED;
     if ((r = run_main(p, m.shape, mode, st))) return r;

@@ -19,7 +19,8 @@
 // per-CTA tables merge into the global one at the end, so every layer
 // configuration yields the same exact groups.  A compaction kernel turns
 // occupied slots into dense output rows (warp ballot / popc, one atomic per
-// warp).  MODE_KEYSET counts distinct keys instead (the exact sizing pass).
+// warp).  Runs the fused filter + aggregate shape (ShapeQ1) and plans with a
+// staging ring of their own; gen.cu and stream.cu have the other shapes.
 #include "groupby.cuh"
 #include "smtab.cuh"
 
@@ -315,28 +316,6 @@ __device__ __noinline__ void gtab_row(const GbParams& p, uint64_t ek, uint64_t v
   Vals<S::A> x;
   S::from_val(val, x);
   gtab_update_inl<S>(p, ek, x);
-}
-
-// Key set for the exact distinct count; false when the set overflowed.
-__device__ __noinline__ bool gset_insert(const GbParams& p, uint64_t ek) {
-  const uint64_t mask = (1ull << p.log2_slots) - 1;
-  uint64_t s = slot_of(ek, p.log2_slots);
-  for (uint32_t i = 0; i < p.max_probe; ++i) {
-    uint64_t k = ld_relaxed(p.tkeys + s);
-    if (k == ek) return true;
-    if (k == 0) {
-      k = atomicCAS((unsigned long long*)(p.tkeys + s), 0ull, (unsigned long long)ek);
-      if (k == 0) {
-        atomicAdd(&p.hdr->aux, 1ull);
-        return true;
-      }
-      if (k == ek) return true;
-    }
-    s = (s + 1) & mask;
-    if ((i & 31) == 31 && ld_relaxed_u32(&p.hdr->overflow)) return false;
-  }
-  atomicOr(&p.hdr->overflow, 1u);
-  return false;
 }
 
 // ---------------------------------------------------------------- backends
@@ -670,41 +649,11 @@ struct BePartScatter {
   __device__ void flush(const GbParams& p) { hot.flush(p); }
 };
 
-// Distinct-key counting: a CTA-shared key filter in front of the global set.
-template <class S>
-struct BeKeySet {
-  static constexpr int A = S::A;
-  static constexpr int ID = relhost::K_GB_KEYSET;
-  static constexpr int SIDE = SIDE_COUNT;
-  uint64_t* tk;
-  __host__ __device__ static uint64_t bytes(uint32_t, uint32_t shared) { return 8ull * shared; }
-  __device__ void bind(uint8_t* area, const GbParams&) { tk = (uint64_t*)area; }
-  __device__ void init(const GbParams& p) {
-    for (uint32_t i = threadIdx.x; i < p.smem_slots; i += GB_BLOCK) tk[i] = 0;
-  }
-  __device__ __forceinline__ bool update(const GbParams& p, uint64_t ek, const Vals<A>&) {
-    const uint32_t mask = p.smem_slots - 1;
-    uint32_t s = small_slot_of(ek, mask, SHARED_MULT);
-    for (uint32_t i = 0; i < p.shared_probes; ++i) {
-      uint64_t k = *(volatile uint64_t*)(tk + s);
-      if (k == ek) return true;  // this CTA already sent the key to the global set
-      if (k == 0) {
-        k = atomicCAS((unsigned long long*)(tk + s), 0ull, (unsigned long long)ek);
-        if (k == 0) break;  // first sight in this CTA
-        if (k == ek) return true;
-      }
-      s = (s + 1) & mask;
-    }
-    return gset_insert(p, ek);
-  }
-  __device__ void flush(const GbParams&) {}
-};
-
 // -------------------------------------------------------------- main kernel
 
 // Fold rows [0, nrows) of a tile view into the backend; returns false once
 // the global table overflowed (later rows are then pointless).
-template <class S, class BE, bool KEYSET, class V>
+template <class S, class BE, class V>
 __device__ __forceinline__ bool run_rows(const GbParams& p, BE& be, const V& v, int nrows) {
   bool ok = true;
   const auto q = S::prep(p, v);
@@ -729,7 +678,7 @@ __device__ __forceinline__ bool run_rows(const GbParams& p, BE& be, const V& v, 
 // "full" when its bytes have landed (full[s]) and "empty" again when all
 // eight consumer warps have arrived on empty[s].  No CTA-wide barrier runs
 // per tile.  Every wait is bounded; a wait that gives up sets hdr->timeout.
-template <class S, class BE, bool KEYSET, bool USE_TMA>
+template <class S, class BE, bool USE_TMA>
 __global__ void __launch_bounds__(GB_THREADS) gb_main(const __grid_constant__ GbParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint64_t* full = (uint64_t*)smem;        // [n_stages]
@@ -797,7 +746,7 @@ __global__ void __launch_bounds__(GB_THREADS) gb_main(const __grid_constant__ Gb
         *(volatile int*)abort_flag = 1;
         break;
       }
-      if (live) live = run_rows<S, BE, KEYSET>(p, be, SmemView{stages + (size_t)s * p.stage_bytes}, (int)T);
+      if (live) live = run_rows<S, BE>(p, be, SmemView{stages + (size_t)s * p.stage_bytes}, (int)T);
       if ((k & 31) == 31) {  // now and then, notice another CTA's overflow
         uint32_t f = lane == 0 ? ld_relaxed_u32(&p.hdr->overflow) : 0;
         live = live && __shfl_sync(0xffffffffu, f, 0) == 0;
@@ -809,13 +758,13 @@ __global__ void __launch_bounds__(GB_THREADS) gb_main(const __grid_constant__ Gb
     }
     const int64_t tail0 = n_tiles * T;
     if (live && tail0 < p.n_rows && blockIdx.x == (unsigned)(n_tiles % gridDim.x))
-      run_rows<S, BE, KEYSET>(p, be, GlobalView{tail0}, (int)(p.n_rows - tail0));
+      run_rows<S, BE>(p, be, GlobalView{tail0}, (int)(p.n_rows - tail0));
   } else {
     for (int64_t k = 0; k < mine; ++k) {
       const int64_t t = (int64_t)blockIdx.x + k * (int64_t)gridDim.x;
       const int64_t r0 = t * T;
       const int nrows = (int)(p.n_rows - r0 < T ? p.n_rows - r0 : T);
-      const bool ok = run_rows<S, BE, KEYSET>(p, be, GlobalView{r0}, nrows);
+      const bool ok = run_rows<S, BE>(p, be, GlobalView{r0}, nrows);
       uint32_t f = lane == 0 ? ld_relaxed_u32(&p.hdr->overflow) : 0;
       f = __shfl_sync(0xffffffffu, f, 0);
       if (!__all_sync(0xffffffffu, ok) || f) break;  // warp-uniform exit
@@ -1229,18 +1178,6 @@ auto with_shape(int shape, F&& f) {
   }
 }
 
-// The key-set pass only needs keys and filters: it runs on a reduced
-// descriptor, so fewer shapes are instantiated for it.
-template <class F>
-auto with_keyset_shape(int shape, F&& f) {
-  switch (shape) {
-    case SHAPE_Q1: return f(ShapeQ1{});
-    case SHAPE_KVRT64: case SHAPE_KV4_64: case SHAPE_KV2_64: return f(ShapeKVRT<int64_t>{});
-    case SHAPE_KVRT32: case SHAPE_KV4_32: case SHAPE_KV2_32: return f(ShapeKVRT<int32_t>{});
-    default: return f(ShapeGeneric{});
-  }
-}
-
 // Partitioned passes: key + int64 value shapes only.
 template <class F>
 auto with_part_shape(int shape, F&& f) {
@@ -1268,16 +1205,16 @@ auto with_regs(int shape, uint32_t ns, F&& f) {
   }
 }
 
-template <class S, class BE, bool KEYSET, bool TMA>
+template <class S, class BE, bool TMA>
 size_t smem_of(const GbParams& p) {
   const uint64_t be = (BE::bytes(p.tiny_slots, p.smem_slots) + 127) & ~127ull;
   return GB_SMEM_HEAD + be + (TMA ? (size_t)p.n_stages * p.stage_bytes : 0);
 }
 
-template <class S, class BE, bool KEYSET, bool TMA>
+template <class S, class BE, bool TMA>
 int occupancy(const GbParams& p) {
-  auto kern = gb_main<S, BE, KEYSET, TMA>;
-  const size_t smem = smem_of<S, BE, KEYSET, TMA>(p);
+  auto kern = gb_main<S, BE, TMA>;
+  const size_t smem = smem_of<S, BE, TMA>(p);
   if (smem > 227 * 1024) return 0;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
@@ -1288,11 +1225,11 @@ int occupancy(const GbParams& p) {
   return per_sm;
 }
 
-template <class S, class BE, bool KEYSET, bool TMA>
+template <class S, class BE, bool TMA>
 rel_status launch_one(const GbParams& p, cudaStream_t st) {
-  auto kern = gb_main<S, BE, KEYSET, TMA>;
-  const size_t smem = smem_of<S, BE, KEYSET, TMA>(p);
-  const int per_sm = occupancy<S, BE, KEYSET, TMA>(p);
+  auto kern = gb_main<S, BE, TMA>;
+  const size_t smem = smem_of<S, BE, TMA>(p);
+  const int per_sm = occupancy<S, BE, TMA>(p);
   if (per_sm < 1) {
     relhost::set_error("group-by: %zu bytes of shared memory per CTA cannot launch", smem);
     return REL_E_UNSUPPORTED;
@@ -1316,7 +1253,6 @@ int gb_shape_width(int shape) {
 }
 
 uint64_t gb_backend_smem_bytes(int mode, int shape, uint32_t tiny_slots, uint32_t smem_slots) {
-  if (mode == MODE_KEYSET) return 8ull * smem_slots;
   if (mode == MODE_PHIST)
     return with_part_shape(shape, [&](auto s) {
       return BePartHist<decltype(s)>::bytes(tiny_slots, smem_slots);
@@ -1337,27 +1273,21 @@ int gb_ctas_per_sm(const GbParams& p, int shape, int mode, bool tma) {
     return with_part_shape(shape, [&](auto s) {
       using S = decltype(s);
       if (mode == MODE_PHIST)
-        return tma ? occupancy<S, BePartHist<S>, false, true>(p)
-                   : occupancy<S, BePartHist<S>, false, false>(p);
-      return tma ? occupancy<S, BePartScatter<S>, false, true>(p)
-                 : occupancy<S, BePartScatter<S>, false, false>(p);
-    });
-  if (mode == MODE_KEYSET)
-    return with_keyset_shape(shape, [&](auto s) {
-      using S = decltype(s);
-      return tma ? occupancy<S, BeKeySet<S>, true, true>(p)
-                 : occupancy<S, BeKeySet<S>, true, false>(p);
+        return tma ? occupancy<S, BePartHist<S>, true>(p)
+                   : occupancy<S, BePartHist<S>, false>(p);
+      return tma ? occupancy<S, BePartScatter<S>, true>(p)
+                 : occupancy<S, BePartScatter<S>, false>(p);
     });
   if (mode == MODE_TINY)
     return with_regs(shape, p.tiny_ns, [&](auto be) {
       using BE = decltype(be);
       using S = typename BE::Shape;
-      return tma ? occupancy<S, BE, false, true>(p) : occupancy<S, BE, false, false>(p);
+      return tma ? occupancy<S, BE, true>(p) : occupancy<S, BE, false>(p);
     });
   return with_shape(shape, [&](auto s) {
     using S = decltype(s);
-    return tma ? occupancy<S, BeLayered<S>, false, true>(p)
-               : occupancy<S, BeLayered<S>, false, false>(p);
+    return tma ? occupancy<S, BeLayered<S>, true>(p)
+               : occupancy<S, BeLayered<S>, false>(p);
   });
 }
 
@@ -1367,27 +1297,21 @@ rel_status gb_launch_main(const GbParams& p, int shape, int mode, bool tma, cuda
     return with_part_shape(shape, [&](auto s) {
       using S = decltype(s);
       if (mode == MODE_PHIST)
-        return tma ? launch_one<S, BePartHist<S>, false, true>(p, st)
-                   : launch_one<S, BePartHist<S>, false, false>(p, st);
-      return tma ? launch_one<S, BePartScatter<S>, false, true>(p, st)
-                 : launch_one<S, BePartScatter<S>, false, false>(p, st);
-    });
-  if (mode == MODE_KEYSET)
-    return with_keyset_shape(shape, [&](auto s) {
-      using S = decltype(s);
-      return tma ? launch_one<S, BeKeySet<S>, true, true>(p, st)
-                 : launch_one<S, BeKeySet<S>, true, false>(p, st);
+        return tma ? launch_one<S, BePartHist<S>, true>(p, st)
+                   : launch_one<S, BePartHist<S>, false>(p, st);
+      return tma ? launch_one<S, BePartScatter<S>, true>(p, st)
+                 : launch_one<S, BePartScatter<S>, false>(p, st);
     });
   if (mode == MODE_TINY)
     return with_regs(shape, p.tiny_ns, [&](auto be) {
       using BE = decltype(be);
       using S = typename BE::Shape;
-      return tma ? launch_one<S, BE, false, true>(p, st) : launch_one<S, BE, false, false>(p, st);
+      return tma ? launch_one<S, BE, true>(p, st) : launch_one<S, BE, false>(p, st);
     });
   return with_shape(shape, [&](auto s) {
     using S = decltype(s);
-    return tma ? launch_one<S, BeLayered<S>, false, true>(p, st)
-               : launch_one<S, BeLayered<S>, false, false>(p, st);
+    return tma ? launch_one<S, BeLayered<S>, true>(p, st)
+               : launch_one<S, BeLayered<S>, false>(p, st);
   });
 }
 

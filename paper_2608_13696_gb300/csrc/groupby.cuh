@@ -15,14 +15,13 @@ constexpr int SHARED_MAX_SLOTS = 4096;
 
 enum GbMode : int {
   MODE_LAYERED = 0,
-  MODE_KEYSET = 1,
   MODE_TINY = 2,
   MODE_PHIST = 3,     // partitioned: count rows per (partition, CTA)
   MODE_PSCATTER = 4   // partitioned: write rows into their partitions
 };
 
 // What a pass does with rows whose key is INT64_MIN (they bypass tables).
-enum SideMode : int { SIDE_AGG = 0, SIDE_COUNT = 1, SIDE_SKIP = 2 };
+enum SideMode : int { SIDE_AGG = 0, SIDE_SKIP = 2 };
 
 // Partitioned group-by record: the stored key and the row's raw value.
 struct alignas(16) PartRec {
@@ -103,7 +102,7 @@ struct GbParams {
   unsigned int* cursor1;    // [2^PART_L1_BITS] next free record of each level-1 bin
   unsigned int* part_extra; // further pieces of oversized partitions (gb_part_scan2)
   unsigned int* l2_tiles;   // [bins + 1] exclusive prefix of the level-2 tiles per bin
-  // global table (or key set in MODE_KEYSET)
+  // global table (or key set)
   uint64_t* tkeys;
   unsigned long long* taggs;  // slots x n_aggs words
   int32_t log2_slots;
@@ -127,9 +126,9 @@ rel_status gb_launch_compact(const GbParams& p, const GbOut& o, cudaStream_t st)
 // offset inside each partition) from the histogram, then per-partition tables.
 rel_status gb_launch_part_scan(const GbParams& p, bool cta_offsets, cudaStream_t st);
 rel_status gb_launch_part_agg(const GbParams& p, int shape, const GbOut& o, cudaStream_t st);
-// Streaming kernel for key/value shapes (stream.cu): pinned keys and/or a
-// small shared table in front of the global table, no staging ring.
-bool gb_stream_eligible(const GbParams& p, int shape, int n_hot);
+// Key/value shapes (stream.cu): pinned keys in front of the global table, a
+// CTA-shared table, or the global table alone; no staging ring.
+bool gb_stream_shape(int shape);
 rel_status gb_launch_stream(const GbParams& p, int shape, cudaStream_t st);
 // Histogram (scatter = false) or scatter pass of the partitioned variant for
 // key/value shapes, streaming; grid = p.fixed_grid CTAs in both passes.

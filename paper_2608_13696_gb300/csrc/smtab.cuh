@@ -88,38 +88,27 @@ __device__ __forceinline__ uint32_t high_with_carry(uint32_t old, uint64_t x) {
   return h;
 }
 
-// NA = 4: sum, count, min, max; NA = 2: sum, count.
-template <int NA>
-struct SmTab {
+// The keys of a table: buckets of two slots.
+struct KeyTab {
   static constexpr uint32_t SPARE = 32;  // slots past the table, one per lane, for idle rows
-  uint32_t mm, key, lo, hi, cnt;         // shared addresses of the arrays
-  uint32_t slots, shift, idle;           // shift = 32 - log2(slots); idle: this lane's spare slot
+  uint32_t key;                          // shared address of the key array (16-byte aligned)
+  uint32_t slots, idle;                  // an even number; this lane's spare slot
 
-  __host__ __device__ static size_t bytes(uint32_t slots) {
-    return (size_t)slots * 8 + (size_t)(slots + SPARE) * (12 + (NA == 4 ? 16 : 0));
-  }
-
-  __device__ __forceinline__ void bind(void* base, uint32_t n) {  // n: a power of two >= 16
+  __device__ __forceinline__ void bind(uint32_t addr, uint32_t n) {
+    key = addr;
     slots = n;
-    shift = (uint32_t)__clz((int)n) + 1;
-    mm = smem_u32(base);
-    key = mm + (NA == 4 ? 16 * (n + SPARE) : 0);
-    lo = key + 8 * n;
-    hi = lo + 4 * (n + SPARE);
-    cnt = hi + 4 * (n + SPARE);
     idle = n + (threadIdx.x & 31);
   }
-  // All threads of the CTA; a barrier must follow.
-  __device__ __forceinline__ void clear() const {
-    for (uint32_t a = mm + 16 * threadIdx.x; a < cnt + 4 * (slots + SPARE); a += 16 * blockDim.x)
-      asm volatile("st.shared.v2.u64 [%0], {%1, %1};" ::"r"(a), "l"(0ull) : "memory");
-  }
-  // First slot of the home bucket: top bits of a multiplicative hash of the
-  // whole key (a packed key's columns sit in different halves, so a folded
-  // 32-bit hash would lay whole families of keys on the same few slots).
+  // First slot of the home bucket, from a multiplicative hash of the whole key
+  // (a packed key's columns sit in different halves, so a folded 32-bit hash
+  // would lay whole families of keys on the same few slots).
   __device__ __forceinline__ uint32_t home(uint64_t ek) const {
-    return ((uint32_t)((ek * 0x9E3779B97F4A7C15ull) >> 32) >> shift) & ~1u;
+    return __umulhi((uint32_t)((ek * 0x9E3779B97F4A7C15ull) >> 32), slots >> 1) << 1;
   }
+  __device__ __forceinline__ uint32_t next(uint32_t s) const {
+    return s + 2 == slots ? 0 : s + 2;
+  }
+  __device__ __forceinline__ uint64_t key_of(uint32_t s) const { return lds64(key + 8 * s); }
 
   // Slots of U keys, inserting the new ones; a key of 0 takes no part and gets
   // the spare slot, as do rows that found no slot within `probes` further
@@ -144,7 +133,7 @@ struct SmTab {
         const bool e0 = k0[j] == ek[j], e1 = k1[j] == ek[j];
         if (!e0 && !e1) {
           miss |= 1u << j;
-          if (k1[j] != 0) s[j] = (s[j] + 2) & (slots - 1);  // the bucket is full
+          if (k1[j] != 0) s[j] = next(s[j]);  // the bucket is full
         }
         if (!e0 && e1) s[j] |= 1;
         if (ek[j] == 0) {
@@ -173,7 +162,7 @@ struct SmTab {
         }
       }
       const bool done = a == k || b == k;
-      w = a == k ? w : b == k ? w + 1 : (w + 2) & (slots - 1);
+      w = a == k ? w : b == k ? w + 1 : next(w);
       if (done) {
         miss ^= bit;
       } else if (--probes <= 0) {
@@ -188,6 +177,34 @@ struct SmTab {
     }
     __syncwarp();
     return left;
+  }
+};
+
+// NA = 4: sum, count, min, max; NA = 2: sum, count.
+template <int NA>
+struct SmTab : KeyTab {
+  uint32_t mm, lo, hi, cnt;  // shared addresses of the word arrays
+
+  __host__ __device__ static size_t bytes(uint32_t slots) {
+    return (size_t)slots * 8 + (size_t)(slots + SPARE) * (12 + (NA == 4 ? 16 : 0));
+  }
+  // The most slots (a multiple of 16) a table of so many bytes holds.
+  __host__ static uint32_t fit(size_t bytes) {
+    const size_t word = 12 + (NA == 4 ? 16 : 0);
+    return (uint32_t)((bytes - SPARE * word) / (8 + word)) & ~15u;
+  }
+
+  __device__ __forceinline__ void bind(void* base, uint32_t n) {  // n: a multiple of 16
+    mm = smem_u32(base);
+    KeyTab::bind(mm + (NA == 4 ? 16 * (n + SPARE) : 0), n);
+    lo = key + 8 * n;
+    hi = lo + 4 * (n + SPARE);
+    cnt = hi + 4 * (n + SPARE);
+  }
+  // All threads of the CTA; a barrier must follow.
+  __device__ __forceinline__ void clear() const {
+    for (uint32_t a = mm + 16 * threadIdx.x; a < cnt + 4 * (slots + SPARE); a += 16 * blockDim.x)
+      asm volatile("st.shared.v2.u64 [%0], {%1, %1};" ::"r"(a), "l"(0ull) : "memory");
   }
 
   // Add rows with values v to the groups of slots s.
@@ -212,7 +229,6 @@ struct SmTab {
     for (int j = 0; j < U; ++j) reds_add_nz(hi + 4 * s[j], high_with_carry(old[j], v[j] + SUM_BIAS));
   }
 
-  __device__ __forceinline__ uint64_t key_of(uint32_t s) const { return lds64(key + 8 * s); }
   // The encoded words of a slot (after a barrier behind the adds).
   __device__ __forceinline__ void words(uint32_t s, uint64_t (&w)[NA]) const {
     const uint32_t c = lds32(cnt + 4 * s);

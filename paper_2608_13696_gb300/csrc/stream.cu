@@ -264,7 +264,7 @@ __device__ __noinline__ void rare_row(const GbParams& p, uint64_t ek, uint64_t v
 // are not used: on a hot key the table's adds serialise over a warp's lanes
 // (15 ns a warp at worst), less than a second lookup costs every row.
 constexpr int SG_U = 4;            // rows per thread per chunk
-constexpr uint32_t SG_MAX_BYTES = 200 * 1024;
+constexpr uint32_t SG_MAX_BYTES = 220 * 1024;
 
 template <class KT, int NA>
 __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbParams p) {
@@ -696,22 +696,31 @@ rel_status launch_rows(K kern, int block, size_t smem, int64_t chunk, const GbPa
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(stream)");
 }
 
+// Pinned keys that gb_stream_k keeps in thread-private words.
+bool pins_fit(const GbParams& p, int na, int n_hot) {
+  return p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= (na == 4 ? pin_max<4>() : pin_max<2>());
+}
+
 template <class KT, int NA>
 rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
-  if (p.smem_slots) {
+  int n_hot = 0;
+  for (uint32_t i = 0; i < p.tiny_slots && p.tiny_frozen; ++i) n_hot += p.tiny_init[i] != 0;
+  if (p.smem_slots || (p.tiny_slots && !pins_fit(p, NA, n_hot))) {
     // 1024 resident threads per SM whatever the table's size; small inputs in
     // small CTAs, so that more SMs take part
     const int64_t small = (int64_t)relhost::device_sms() * 2048;
     GbParams q = p;
-    // a plan's table is half full; where the rows pay for clearing and merging
-    // it, up to four times the slots keep more keys in their home bucket (1e8
-    // rows, 400 groups: 1024 slots 0.64 ms, 4096 slots 0.50 ms), as long as two
-    // CTAs fit -- and a table that would be nearly full is doubled once more
+    // A plan's table is half full (with first-come or too many pinned
+    // thread-private slots instead: its few groups in 256 slots).  Where the
+    // rows pay for clearing and merging it, up to four times the slots keep
+    // more keys in their home bucket (1e8 rows, 400 groups: 1024 slots 0.64
+    // ms, 4096 slots 0.50 ms), as long as two CTAs fit; a plan at the largest
+    // table gets what one CTA per SM can hold.
+    if (q.smem_slots < 256) q.smem_slots = 256;
     if (p.n_rows > 8 * small)
       while (q.smem_slots < 4 * p.smem_slots && SmTab<NA>::bytes(2 * q.smem_slots) <= 110 * 1024)
         q.smem_slots *= 2;
-    if (NA == 2 && q.smem_slots == SHARED_MAX_SLOTS && q.smem_slots == p.smem_slots)
-      q.smem_slots *= 2;
+    if (p.smem_slots == SHARED_MAX_SLOTS) q.smem_slots = SmTab<NA>::fit(SG_MAX_BYTES);
     const size_t smem = SmTab<NA>::bytes(q.smem_slots);
     const int block = smem > 110 * 1024 ? 1024 : smem > 54 * 1024 || p.n_rows > small ? 512 : 256;
     return launch_rows(gb_smem_k<KT, NA>, block, smem, (int64_t)block * SG_U, q, st);
@@ -724,18 +733,9 @@ rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
 
 }  // namespace
 
-bool gb_stream_eligible(const GbParams& p, int shape, int n_hot) {
-  const bool kv = shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
-                  shape == SHAPE_KV2_32;
-  if (!kv) return false;
-  const int na = (shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32) ? 4 : 2;
-  // a CTA-shared table: gb_smem_k
-  if (p.smem_slots)
-    return (na == 4 ? SmTab<4>::bytes(p.smem_slots) : SmTab<2>::bytes(p.smem_slots)) <= SG_MAX_BYTES;
-  // thread-private slots only when pinned (a first-come thread-private
-  // table is the fused kernel's job)
-  const int pmax = na == 4 ? pin_max<4>() : pin_max<2>();
-  return !p.tiny_slots || (p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= pmax);
+bool gb_stream_shape(int shape) {
+  return shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
+         shape == SHAPE_KV2_32;
 }
 
 // Level 2 of the streaming scatter: every tile of PART_TILE level-1 records
@@ -880,9 +880,7 @@ uint32_t gb_ppass_stream_grid(const GbParams& p, int shape, uint32_t cap) {
 }
 
 bool gb_ppass_stream_eligible(const GbParams& p, int shape, int n_hot) {
-  const bool kv = shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
-                  shape == SHAPE_KV2_32;
-  if (!kv || p.fixed_grid < 1) return false;
+  if (!gb_stream_shape(shape) || p.fixed_grid < 1) return false;
   const int na = (shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32) ? 4 : 2;
   const int pmax = na == 4 ? pin_max<4>() : pin_max<2>();
   if (p.tiny_slots && !(p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= pmax)) return false;
