@@ -1532,6 +1532,8 @@ rel_status rel_groupby_agg(const rel_groupby_desc* d, const rel_plan* plan, void
   } else if (!plan->tile_rows && (m.shape == SHAPE_GENERIC || m.shape == SHAPE_KVRT64 ||
                                   m.shape == SHAPE_KVRT32)) {
     if ((r = gb_launch_gen(p, plan->est_groups, st))) return r;
+  } else if (!plan->tile_rows && m.shape == SHAPE_Q1 && gb_q1_eligible(p, plan->n_hot)) {
+    if ((r = gb_launch_q1(p, plan->n_hot, st))) return r;
   } else {
     const int mode = p.tiny_ns ? MODE_TINY : MODE_LAYERED;
     if ((r = run_main(p, m.shape, mode, st))) return r;

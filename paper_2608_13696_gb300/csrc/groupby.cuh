@@ -126,6 +126,9 @@ rel_status gb_launch_compact(const GbParams& p, const GbOut& o, cudaStream_t st)
 // offset inside each partition) from the histogram, then per-partition tables.
 rel_status gb_launch_part_scan(const GbParams& p, bool cta_offsets, cudaStream_t st);
 rel_status gb_launch_part_agg(const GbParams& p, int shape, const GbOut& o, cudaStream_t st);
+// ShapeQ1 with every group pinned (q1.cu).
+bool gb_q1_eligible(const GbParams& p, int n_hot);
+rel_status gb_launch_q1(const GbParams& p, int n_hot, cudaStream_t st);
 // Key/value shapes (stream.cu): pinned keys in front of the global table, a
 // CTA-shared table, or the global table alone; no staging ring.
 bool gb_stream_shape(int shape);

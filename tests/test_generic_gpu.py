@@ -71,3 +71,33 @@ def test_layers_and_overflow(smem, variant):
     with pytest.raises(rel.RelError) as e:
         rel.groupby(qc, plan=p)
     assert e.value.status == rel.REL_E_OVERFLOW
+
+
+@pytest.mark.parametrize("n", [1, 3, 1023, 3073, 700_001])
+@pytest.mark.parametrize("pins", [1, 3, 6])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_fused_shape_with_pinned_groups(n, pins, offset):
+    """All groups pinned, some pinned (the others take the global table), rows
+    around the chunk edges, unaligned columns, extreme values."""
+    import synth
+    from paper_2608_13696_gb300 import workloads
+
+    li = synth.lineitem(n + offset, seed=n + pins)
+    li["price"][:: 97] = I64.max
+    li["qty"][1:: 89] = I64.min
+    q = oracle.lineitem_query({k: v[offset:] for k, v in li.items()})
+    ek, ea = oracle.groupby(q)
+    qc = workloads.lineitem_query({k: cuda(v)[offset:] for k, v in li.items()})
+    p = rel.plan_groupby(qc, groups_hint=6).layers(8, 0, rel.VAR_SMEM)
+    keys = [0, 1, 256, 257, 512, 513][:pins]
+    for mult in range(0x9E3779B1, 0x9E3779B1 + 2 * 4096, 2):  # a multiplier without collisions
+        f = [((((k ^ (1 << 31)) & 0xFFFFFFFF) * (mult & 0xFFFFFFFF)) >> 32) & 7 for k in keys]
+        if len(set(f)) == len(f):
+            break
+    p.tiny_mult = mult & 0xFFFFFFFF
+    p.n_hot = len(keys)
+    for i, k in enumerate(keys):
+        p.hot_keys[i] = k
+    gk, ga = canon_groupby(*rel.groupby(qc, plan=p))
+    np.testing.assert_array_equal(gk, ek)
+    np.testing.assert_array_equal(ga, ea)
