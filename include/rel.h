@@ -192,7 +192,7 @@ typedef struct {
  *      rel_sketch, then the registered planner network (rel_planner_set) on
  *      its features; est_groups = max(ceil(1.25 * 2^(y0 + 1)), sample distinct
  *      keys), the variant is the network's most likely one that the
- *      descriptor supports.  For one int32 / int64 key without a filter,
+ *      descriptor supports (REL_VAR_GLOBAL: left to the rule by group count).  For one int32 / int64 key without a filter,
  *      at least 2^22 rows, and a sample whose distinct keys were more than
  *      3/4 seen once (a long tail the sample cannot size), one streaming
  *      pass of a full-data HyperLogLog (4096 registers) gives est = its

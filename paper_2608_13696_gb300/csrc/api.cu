@@ -417,6 +417,10 @@ constexpr uint32_t PART_MAX_GRID = PART_HIST_COLS - 1;  // CTAs of the histogram
 // records into equal pieces instead of taking whole partitions: 256
 // partitions would occupy 256 of its ~600 CTAs.
 constexpr int PART_SPLIT_BITS = 8;
+// the most groups that 256 partitions (one scatter level) take, 1172 to a
+// 2048-slot table (four aggregates, 250000
+// groups: 2.5e7 rows 0.69 -> 0.56 ms, 1e8 2.43 -> 1.86)
+constexpr int64_t PART_ONE_LEVEL_GROUPS = 300000;
 
 bool part_shape(int shape) {
   return shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
@@ -519,6 +523,9 @@ void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
   uint64_t per = (uint64_t)(est / 768);
   int bits = 4;
   while (bits < PART_MAX_BITS && (1ull << bits) < per) ++bits;
+  // a little past one scatter level: larger tables instead of the second level
+  const bool larger = bits == PART_L1_BITS + 1 && est <= PART_ONE_LEVEL_GROUPS;
+  if (larger) bits = PART_L1_BITS;
   plan->variant = REL_VAR_PARTITIONED;
   plan->part_bits = bits;
   // each partition's table at load <= 0.5 on average (the partitions' key
@@ -527,6 +534,7 @@ void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
   const uint64_t keys_per_part = (uint64_t)est >> bits;
   plan->smem_slots = (int32_t)next_pow2(keys_per_part * 2 < 256 ? 256 : keys_per_part * 2);
   if (plan->smem_slots > SHARED_MAX_SLOTS) plan->smem_slots = SHARED_MAX_SLOTS;
+  if (larger) plan->smem_slots = 2048;
   plan->tiny_slots = 0;     // pinned heavy hitters only (from a sketch)
   // spill table: a partition whose keys do not all fit its table sends all
   // of them to the global table.  Sized for a quarter of the keys while the
@@ -553,7 +561,7 @@ void choose_layers(int64_t est, int words, rel_plan* plan) {
   } else if (est <= 24 && words <= 2) {
     plan->variant = REL_VAR_SMEM;
     plan->tiny_slots = 32;
-  } else if (est <= (words == 2 ? 4096 : 2048)) {
+  } else if (est <= (words == 2 ? 5120 : words == 4 ? 3072 : 2048)) {
     plan->variant = REL_VAR_SMEM;
     plan->tiny_slots = words <= 6 ? 8 : 0;  // catches a skewed input's hottest keys
     plan->smem_slots = (int32_t)next_pow2((uint64_t)(2 * est));
@@ -638,6 +646,21 @@ void apply_sketch(const rel_sketch_info& s, int words, rel_plan* plan) {
   }
 }
 
+// A partitioned plan's input is better off in one global table: few rows, which
+// do not make up for the partition passes' launches, and no key so frequent --
+// overall or in runs -- that its rows would queue up on one address.  (Uniform
+// keys, four aggregates, 20000 groups: 1e6 rows 42 against 93 us, 6e6 147
+// against 174, 2.5e7 550 against 434; 4000 groups cross over at 4e6 rows.)
+// Fewer groups than 8192 queue up on their slots, more than a quarter of the
+// rows make a table that takes longer to clear and scan.
+constexpr int64_t GLOBAL_MAX_ROWS = 1ll << 22;
+
+bool prefer_global(const rel_sketch_info& s, int64_t n_rows, const rel_plan* plan) {
+  return plan->variant == REL_VAR_PARTITIONED && plan->n_hot == 0 && plan->tiny_slots == 0 &&
+         n_rows <= GLOBAL_MAX_ROWS && plan->est_groups >= 8192 &&
+         4 * plan->est_groups <= n_rows && s.runs > 0 && s.kept < 4 * s.runs;
+}
+
 // Probe limits of the per-CTA layers: a layer that must hold every group
 // scans it all; a cache in front of a larger layer gives up early.  Pinned
 // hot keys sit at their own hash slot, so one probe decides.
@@ -656,6 +679,7 @@ rel_status set_layers(GbParams& p, const rel_plan* plan, int shape) {
              REL_E_INVALID;
     p.tiny_frozen = 1;
     p.tiny_probes = 1;
+    p.all_pinned = tiny_only;
     // at most four pinned keys, no CTA-shared layer, a shape of <= 5 words:
     // keep the accumulators in registers (dense ids in slot order).  With
     // more keys the register file costs more than it saves: 1e8 lineitem
@@ -748,9 +772,6 @@ constexpr uint64_t EXACT_SET_L2_SLOTS = 1ull << 24;
 // the only one probed, and the random bucket reads still mostly hit L2 while
 // the column streams past
 constexpr uint64_t EXACT_SET_FIRST_BYTES = 256ull << 20;
-// entries of the streaming distinct count's per-CTA filter (0: none; the
-// buckets of frequent keys are served by L1 instead)
-constexpr uint32_t EXACT_FILTER_SLOTS = 0;
 
 // Scratch after the sketch's: the 264 features and the 4 network outputs.
 constexpr uint64_t LEARN_OUT_OFF = 1280;
@@ -792,26 +813,17 @@ rel_status learned_estimate(const rel_groupby_desc* d, bool p_ok, void* ws, size
   const uint64_t sk = rel_sketch_ws_bytes();
   rel_status r = rel_sketch(d, ws, ws_bytes, info, st);
   if (r) return r;
-  float* dx = (float*)((uint8_t*)ws + sk);
-  float* dy = (float*)((uint8_t*)ws + sk + LEARN_OUT_OFF);
-  cudaError_t e = cudaMemcpyAsync(dx, info->features, sizeof info->features,
-                                  cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemcpyAsync");
-  if ((r = mlp_forward(g_planner_bf16, g_planner_f32, dx, 1, dy, nullptr, st))) return r;
-  float y[REL_MLP_OUT];
-  e = cudaMemcpyAsync(y, dy, sizeof y, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return relhost::cuda_fail(e, "reading the planner output");
-  learned_rule(*info, y, d->n_rows, p_ok, est, variant);
   // A 4096-row sample says little about a long tail: when most keys it saw
   // occurred once and the input is large, one streaming pass of a full-data
   // HyperLogLog (about a fifth of the exact count's cost) sizes the table
   // instead -- standard error 1.6 %, sized with 25 % headroom -- and the
-  // variant follows the rule by group count for that size.
+  // variant follows the rule by group count for that size; the network, whose
+  // answer would not be used, is not asked.
   const bool stream_key = d->n_keys == 1 && d->n_preds == 0 &&
                           (d->cols[d->key_cols[0]].type == REL_I64 ||
                            d->cols[d->key_cols[0]].type == REL_I32);
   if (hll_sized) *hll_sized = false;
+  cudaError_t e;
   if (stream_key && d->n_rows >= LEARN_HLL_MIN_ROWS && 4ll * info->singletons > 3ll * info->ndv) {
     uint32_t* dregs = (uint32_t*)((uint8_t*)ws + sk + LEARN_HLL_OFF);
     e = cudaMemsetAsync(dregs, 0, 4ull * HLL_REGS, st);
@@ -829,7 +841,19 @@ rel_status learned_estimate(const rel_groupby_desc* d, bool p_ok, void* ws, size
     *est = n;
     *variant = 0;  // the rule by group count
     if (hll_sized) *hll_sized = true;
+    return REL_OK;
   }
+  float* dx = (float*)((uint8_t*)ws + sk);
+  float* dy = (float*)((uint8_t*)ws + sk + LEARN_OUT_OFF);
+  e = cudaMemcpyAsync(dx, info->features, sizeof info->features,
+                                  cudaMemcpyHostToDevice, st);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemcpyAsync");
+  if ((r = mlp_forward(g_planner_bf16, g_planner_f32, dx, 1, dy, nullptr, st))) return r;
+  float y[REL_MLP_OUT];
+  e = cudaMemcpyAsync(y, dy, sizeof y, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "reading the planner output");
+  learned_rule(*info, y, d->n_rows, p_ok, est, variant);
   return REL_OK;
 }
 
@@ -866,43 +890,72 @@ void choose_variant(int variant, int64_t est, int64_t n_rows, int words, bool p_
   }
 }
 
+// A sample sketch taken together with an exact distinct count: its result
+// stands between the status header and the key set, the two kernels run beside
+// each other, and one copy brings both back.
+struct ExactSketch {
+  const SketchParams* params = nullptr;  // null: no sketch wanted
+  DevSketch out;
+};
+constexpr uint64_t EXACT_SKETCH_BYTES = (sizeof(DevSketch) + 255) & ~(uint64_t)255;
+
+// Clear header and key set, then the sketch.
+rel_status exact_begin(void* ws, uint64_t set_bytes, const ExactSketch* sk, cudaStream_t st) {
+  const uint64_t gap = sk ? EXACT_SKETCH_BYTES : 0;
+  const cudaError_t e = cudaMemsetAsync(ws, 0, HEADER_BYTES + gap + set_bytes, st);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemsetAsync");
+  return sk ? sketch_launch(*sk->params, (DevSketch*)((uint8_t*)ws + HEADER_BYTES), st) : REL_OK;
+}
+
+rel_status exact_end(const void* ws, HostHeader* h, ExactSketch* sk, cudaStream_t st) {
+  if (!sk) return read_header(ws, h, st);
+  uint8_t both[HEADER_BYTES + sizeof(DevSketch)];
+  cudaError_t e = cudaMemcpyAsync(both, ws, sizeof both, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return relhost::cuda_fail(e, "reading the status header");
+  std::memcpy(h, both, sizeof *h);
+  std::memcpy(&sk->out, both + HEADER_BYTES, sizeof sk->out);
+  return REL_OK;
+}
+
 // The exact distinct count of one int32 / int64 key column (no filter) in
 // workspace ws of HEADER_BYTES + 8 * set_slots bytes.  First one pass with a
 // key set of at most EXACT_SET_FIRST_BYTES (load <= ~0.5 up to 1.6e7 distinct
 // keys; its random reads mostly hit L2); when the distinct keys overflow it,
 // the whole workspace is split into K sets of at most EXACT_SET_FIRST_BYTES
 // each (K <= 16) and K passes each count the keys of one hash range.  Every
-// attempt gives the same count.
+// attempt gives the same count.  sk (or null): a sketch to take with the first
+// attempt.
 rel_status exact_distinct(const void* keys, int32_t key_type, int64_t n_rows, void* ws,
-                          uint64_t set_slots, int64_t* est, cudaStream_t st) {
+                          uint64_t set_slots, ExactSketch* sk, int64_t* est, cudaStream_t st) {
   DistinctParams dp;
   std::memset(&dp, 0, sizeof dp);
   dp.keys = keys;
   dp.n_rows = n_rows;
   dp.hdr = (WsHeader*)ws;
-  dp.filter_slots = EXACT_FILTER_SLOTS;
   const uint64_t total_buckets = set_slots / DS_BUCKET_SLOTS;  // set_slots >= 16
   const uint64_t first_buckets = EXACT_SET_FIRST_BYTES / (8ull * DS_BUCKET_SLOTS);
   for (int attempt = 0; attempt < 2; ++attempt) {
     uint32_t passes = 1;
-    uint64_t buckets = total_buckets < first_buckets ? total_buckets : first_buckets;
+    // (the sketch takes its room from the set: 24 of at least 4096 buckets)
+    const uint64_t gap = attempt == 0 && sk ? EXACT_SKETCH_BYTES : 0;
+    uint64_t buckets = std::min(total_buckets - gap / (8 * DS_BUCKET_SLOTS), first_buckets);
     if (attempt == 1) {
-      if (total_buckets <= first_buckets) break;  // the first set was already the full one
+      if (total_buckets <= first_buckets && !sk) break;  // the first set was already the full one
       passes = (uint32_t)std::min<uint64_t>(16, (total_buckets + first_buckets - 1) / first_buckets);
       buckets = total_buckets / passes;
     }
-    cudaError_t e = cudaMemsetAsync(ws, 0, HEADER_BYTES + 8ull * DS_BUCKET_SLOTS * buckets * passes, st);
-    if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemsetAsync");
     rel_status r;
+    if ((r = exact_begin(ws, 8ull * DS_BUCKET_SLOTS * buckets * passes, gap ? sk : nullptr, st))) return r;
     for (uint32_t k = 0; k < passes; ++k) {
       dp.n_pass = passes;
       dp.pass = k;
       dp.n_buckets = buckets;
-      dp.set = (uint64_t*)((uint8_t*)ws + HEADER_BYTES) + (uint64_t)k * buckets * DS_BUCKET_SLOTS;
-      if ((r = distinct_launch(dp, key_type, st))) return r;
+      dp.set = (uint64_t*)((uint8_t*)ws + HEADER_BYTES + gap) + (uint64_t)k * buckets * DS_BUCKET_SLOTS;
+      if ((r = distinct_launch(dp, key_type, gap != 0, st))) return r;
     }
     HostHeader h;
-    if ((r = read_header(ws, &h, st))) return r;
+    if ((r = exact_end(ws, &h, gap ? sk : nullptr, st))) return r;
     if (h.overflow) continue;
     *est = (int64_t)h.aux + (h.n_side > 0 ? 1 : 0);
     return REL_OK;
@@ -957,7 +1010,22 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
     }
     if (d->n_rows == 0) {
       est = 0;
+    } else if ((flags & REL_PLAN_SKETCH) && d->n_rows <= SKETCH_SAMPLE &&
+               plan->scratch_bytes >= rel_sketch_ws_bytes()) {
+      // the sketch's sample is every row: its distinct keys are the count
+      if ((r = rel_sketch(d, ws, ws_bytes, &info, st))) return r;
+      have_info = true;
+      est = info.ndv;
     } else {
+      ExactSketch both;
+      SketchParams sp;
+      int bits = 0;
+      ExactSketch* sk = nullptr;
+      if ((flags & REL_PLAN_SKETCH) && d->n_rows > SKETCH_SAMPLE) {
+        bits = sketch_params(d, &sp);
+        both.params = &sp;
+        sk = &both;
+      }
       // reduced descriptor: the key and filter columns, one COUNT
       rel_col cols[REL_MAX_COLS];
       int32_t keys[REL_MAX_KEYS];
@@ -991,27 +1059,27 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
       const int ident[REL_MAX_AGGS] = {0, 1, 2, 3, 4, 5, 6, 7};
       fill_params(&kd, ident, kp);
       kp.hdr = (WsHeader*)ws;
-      kp.tkeys = (uint64_t*)((uint8_t*)ws + HEADER_BYTES);
       const int32_t kt = kd.cols[keys[0]].type;
       const bool stream_keys = !(flags & REL_PLAN_GENERIC) && kd.n_keys == 1 &&
                                kd.n_preds == 0 && (kt == REL_I64 || kt == REL_I32);
       if (stream_keys) {
-        r = exact_distinct(kd.cols[keys[0]].data, kt, d->n_rows, ws, set_slots, &est, st);
+        r = exact_distinct(kd.cols[keys[0]].data, kt, d->n_rows, ws, set_slots, sk, &est, st);
         if (r) return r;
       } else {
         // First a key set of at most EXACT_SET_L2_SLOTS slots (128 MB: the
-        // memset is small); only when the distinct keys overflow it, the full
-        // 2 x rows set.  Both give the same count.
-        uint64_t try_slots = set_slots < EXACT_SET_L2_SLOTS ? set_slots : EXACT_SET_L2_SLOTS;
-        for (;;) {
+        // memset is small) and, with a sketch in front of it, of half the
+        // workspace; only when the distinct keys overflow it, the full 2 x rows
+        // set.  Both give the same count.
+        uint64_t try_slots = std::min(sk ? set_slots / 2 : set_slots, EXACT_SET_L2_SLOTS);
+        for (bool first = true;; first = false) {
+          ExactSketch* with = first ? sk : nullptr;
           kp.log2_slots = log2_pow2(try_slots);
           kp.max_probe = (uint32_t)(try_slots < 4096 ? try_slots : 4096);
-          cudaError_t e = cudaMemsetAsync(ws, 0, HEADER_BYTES + 8ull * try_slots, st);
-          if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaMemsetAsync");
-          if ((r = gb_launch_gen_set(kp, st))) return r;
+          kp.tkeys = (uint64_t*)((uint8_t*)ws + HEADER_BYTES + (with ? EXACT_SKETCH_BYTES : 0));
+          if ((r = exact_begin(ws, 8ull * try_slots, with, st))) return r;
+          if ((r = gb_launch_gen_set(kp, with != nullptr, st))) return r;
           HostHeader h;
-          if ((r = read_header(ws, &h, st))) return r;
-          if (h.timeout) return set_error("plan: a device wait timed out"), REL_E_TIMEOUT;
+          if ((r = exact_end(ws, &h, with, st))) return r;
           if (h.overflow && try_slots < set_slots) {
             try_slots = set_slots;
             continue;
@@ -1021,14 +1089,19 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
           break;
         }
       }
+      if (sk) {
+        sketch_fill(d, both.out, bits, &info);
+        have_info = true;
+      }
     }
   } else {
     est = d->n_rows;
   }
   plan->est_groups = est;
   plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
-  choose_variant(forced ? forced : learned, est, d->n_rows, gb_shape_width(m.shape), p_ok, plan);
-  plan->workspace_bytes = plan_ws_bytes(plan, d->n_aggs, d->n_rows);
+  // (a network that prefers the global table leaves the choice to the rules)
+  choose_variant(forced ? forced : learned == REL_VAR_GLOBAL ? 0 : learned, est, d->n_rows,
+                 gb_shape_width(m.shape), p_ok, plan);
   if ((flags & REL_PLAN_SKETCH) && d->n_rows > 0) {
     if (!have_info) {
       const uint64_t need = rel_sketch_ws_bytes();
@@ -1041,7 +1114,13 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
       if ((r = rel_sketch(d, ws, ws_bytes, &info, st))) return r;
     }
     apply_sketch(info, gb_shape_width(m.shape), plan);
+    if (!forced && prefer_global(info, d->n_rows, plan)) {
+      plan->variant = REL_VAR_GLOBAL;
+      plan->part_bits = plan->smem_slots = plan->tiny_slots = 0;
+      plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
+    }
   }
+  plan->workspace_bytes = plan_ws_bytes(plan, d->n_aggs, d->n_rows);
   return REL_OK;
 }
 

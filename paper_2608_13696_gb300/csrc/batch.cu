@@ -108,15 +108,8 @@ __device__ __forceinline__ void side_update(const BatchGb& g, BatchStatus* st, c
 // keys, 32 bytes): one 256-bit load shows four slots for the price of one, so
 // at most half load 97 of 100 rows end at their first load.
 __device__ __forceinline__ uint64_t home_slot(const BatchGb& g, uint64_t ek) {
-  return slot_of(ek, g.log2_slots) & ~3ull;
+  return home_sector(ek, g.log2_slots);
 }
-__device__ __forceinline__ void ld_sector(const uint64_t* p, uint64_t (&k)[4]) {
-  asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
-               : "=l"(k[0]), "=l"(k[1]), "=l"(k[2]), "=l"(k[3])
-               : "l"(p)
-               : "memory");
-}
-
 // Slot of ek at or after slot s (the first of a sector), claiming the first
 // empty one; ~0 when the table overflowed.  Out of line: the rare path.
 __device__ __noinline__ uint64_t global_claim(const BatchGb& g, BatchStatus* st, uint64_t ek,
@@ -335,7 +328,7 @@ __device__ __noinline__ void global_rows(const BatchGb& g, BatchStatus* st, long
 #pragma unroll
       for (int j = 0; j < U; ++j) {
         const uint64_t e = ek[j];
-        const uint32_t at = k[j][0] == e ? 0 : k[j][1] == e ? 1 : k[j][2] == e ? 2 : k[j][3] == e ? 3 : 4;
+        const uint32_t at = in_sector(k[j], e);
         if (at == 4) {
           miss |= 1u << j;
           if (k[j][3] != 0) s[j] = (s[j] + 4) & mask;  // the home sector is full
@@ -354,15 +347,8 @@ __device__ __noinline__ void global_rows(const BatchGb& g, BatchStatus* st, long
       const uint64_t e = second ? ek[1] : ek[0];
       uint64_t w = second ? s[1] : s[0], k[4];
       ld_sector(tk + w, k);
-      uint32_t at = k[0] == e ? 0 : k[1] == e ? 1 : k[2] == e ? 2 : k[3] == e ? 3 : 4;
-      if (at == 4 && k[3] == 0) {  // room as loaded: claim the first empty slot
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (at != 4 || k[q] != 0) continue;
-          const uint64_t old = atomicCAS((unsigned long long*)(tk + w + q), 0ull, (unsigned long long)e);
-          if (old == 0 || old == e) at = q;
-        }
-      }
+      uint32_t at = in_sector(k, e);
+      if (at == 4 && k[3] == 0) at = claim_in_sector(tk + w, k, e);  // room as loaded
       bool done = at != 4;
       w = done ? w + at : (w + 4) & mask;
       if (!done && ((i & 31) == 28 && ld_relaxed_u32(&st->overflow))) {  // already overflowed
@@ -437,7 +423,7 @@ __device__ __forceinline__ void build_tile(const BatchJoin& J, BatchStatus* st, 
     }
 #pragma unroll
     for (int j = 0; j < BUILD_U; ++j) {
-      s[j] = slot_of(ek[j], J.log2_slots) & ~3ull;
+      s[j] = home_sector(ek[j], J.log2_slots);
       got[j] = 1;
       if (ek[j] != 0)
         got[j] = atomicCAS((unsigned long long*)(J.tkeys + s[j]), 0ull, (unsigned long long)ek[j]);
@@ -573,7 +559,7 @@ __device__ __forceinline__ void probe_rows(const BatchJoin& J, BatchStatus* st, 
     }
 #pragma unroll
     for (int j = 0; j < PROBE_U; ++j) {
-      s[j] = slot_of(ek[j], J.log2_slots) & ~3ull;
+      s[j] = home_sector(ek[j], J.log2_slots);
       m[j] = 0;
       bool last = true;
       if (ek[j] != 0) m[j] = match_sector(J.tkeys, s[j], ek[j], &last);

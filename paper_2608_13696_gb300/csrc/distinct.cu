@@ -14,9 +14,9 @@
 //    load, so almost every probe resolves in one L2 request and one compare
 //    chain (the paper's recommendation: fewer instructions per memory
 //    access);
-//  * an optional per-CTA direct-mapped filter of recently sent keys in shared
-//    memory drops repeats before they reach the set (off by default: the
-//    buckets of frequent keys come from L1 anyway);
+//  * the buckets of frequent keys come from L1 (a CTA-private filter of seen
+//    keys in front of it costs more L1 than it saves: 2e8 Zipf rows 1.17 ->
+//    1.45 ms);
 //  * every thread issues the bucket loads of several unfiltered rows before
 //    resolving any (memory-level parallelism), and the kernel runs at high
 //    occupancy so that many chunks of keys are in flight per SM;
@@ -40,9 +40,16 @@ namespace {
 
 constexpr int DS_BLOCK = 256;
 constexpr int DS_U = 8;      // keys per thread per chunk
-constexpr int DS_GROUP = 4;  // keys whose home buckets are in flight together
+constexpr int DS_GROUP = 2;  // keys whose home buckets are in flight together (2 in four CTAs per
+                             // SM, 4 in three: 1.07 and 1.15 ms on 2e8 Zipf rows)
 
 __device__ __forceinline__ uint64_t ds_hash(uint64_t ek) { return ek * 0x9E3779B97F4A7C15ull; }
+
+// Home bucket: the hash's high half scaled to the buckets (fewer than 2^31),
+// one 32-bit multiplication.
+__device__ __forceinline__ uint64_t ds_home(uint64_t ek, uint64_t n_buckets) {
+  return __umulhi((uint32_t)(ds_hash(ek) >> 32), (uint32_t)n_buckets);
+}
 
 // Pass of a key under an n-way hash split (a multiplier independent of ds_hash).
 __device__ __forceinline__ uint32_t ds_pass(uint64_t ek, uint32_t n_pass) {
@@ -154,16 +161,11 @@ struct DsMiss {
 constexpr int DS_WARPS = DS_BLOCK / 32;
 constexpr int DS_QUEUE = 32 * DS_U;  // every row of a warp's chunk
 
-template <class KT, bool FILTER>
-__global__ void __launch_bounds__(DS_BLOCK, 3) distinct_k(const __grid_constant__ DistinctParams p) {
-  extern __shared__ __align__(16) uint64_t filt[];
+template <class KT, bool SPLIT>
+__global__ void __launch_bounds__(DS_BLOCK, 4) distinct_k(const __grid_constant__ DistinctParams p) {
   __shared__ DsMiss queue[DS_WARPS][DS_QUEUE];
   const int lane = threadIdx.x & 31;
   DsMiss* const wq = queue[threadIdx.x >> 5];
-  const uint32_t fmask = p.filter_slots - 1;
-  if (FILTER)
-    for (uint32_t i = threadIdx.x; i < p.filter_slots; i += DS_BLOCK) filt[i] = 0;
-  __syncthreads();
   const KT* keys = (const KT*)p.keys;
   const int64_t n = p.n_rows;
   constexpr int64_t CH = (int64_t)DS_BLOCK * DS_U;
@@ -186,12 +188,7 @@ __global__ void __launch_bounds__(DS_BLOCK, 3) distinct_k(const __grid_constant_
         side += p.pass == 0;
         continue;
       }
-      if (p.n_pass > 1 && ds_pass(ek[j], p.n_pass) != p.pass) continue;
-      if (FILTER) {
-        uint64_t* f = filt + ((uint32_t)(ds_hash(ek[j]) >> 24) & fmask);
-        if (*f == ek[j]) continue;  // this CTA has sent the key already
-        *f = ek[j];
-      }
+      if (SPLIT && ds_pass(ek[j], p.n_pass) != p.pass) continue;
       need |= 1u << j;
     }
     // home buckets of DS_GROUP keys in flight together, then resolved; a
@@ -203,7 +200,7 @@ __global__ void __launch_bounds__(DS_BLOCK, 3) distinct_k(const __grid_constant_
       uint64_t s[DS_GROUP][DS_BUCKET_SLOTS];
 #pragma unroll
       for (int q = 0; q < DS_GROUP; ++q) {
-        const uint64_t b = __umul64hi(ds_hash(ek[g + q]), p.n_buckets);
+        const uint64_t b = ds_home(ek[g + q], p.n_buckets);
         if (need >> (g + q) & 1) ld_bucket(p.set + b * DS_BUCKET_SLOTS, s[q], pol);
       }
 #pragma unroll
@@ -226,7 +223,7 @@ __global__ void __launch_bounds__(DS_BLOCK, 3) distinct_k(const __grid_constant_
       at -= nm;
 #pragma unroll
       for (int j = 0; j < DS_U; ++j)
-        if (miss >> j & 1) wq[at++] = DsMiss{ek[j], __umul64hi(ds_hash(ek[j]), p.n_buckets)};
+        if (miss >> j & 1) wq[at++] = DsMiss{ek[j], ds_home(ek[j], p.n_buckets)};
       __syncwarp();
       for (uint32_t i = lane; i < total; i += 32) {
         const int r = ds_insert(p, wq[i].key, wq[i].bucket);
@@ -249,6 +246,7 @@ __global__ void __launch_bounds__(DS_BLOCK, 3) distinct_k(const __grid_constant_
     if (claims) atomicAdd(&p.hdr->aux, claims);
     if (side) atomicAdd(&p.hdr->n_side, side);
   }
+  wait_for_earlier_kernels();
 }
 
 // The MurmurHash3 64-bit finalizer (Appleby): a bijective mix of the key.
@@ -289,24 +287,21 @@ __global__ void __launch_bounds__(DS_BLOCK) hll_k(const KT* __restrict__ keys, i
     if (r[i]) atomicMax(regs + i, r[i]);
 }
 
-template <class KT, bool FILTER>
-rel_status launch(const DistinctParams& p, cudaStream_t st) {
-  auto kern = distinct_k<KT, FILTER>;
-  const size_t smem = FILTER ? distinct_smem_bytes(p.filter_slots) : 0;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(distinct)");
+template <class KT, bool SPLIT>
+rel_status launch(const DistinctParams& p, bool beside, cudaStream_t st) {
+  auto kern = distinct_k<KT, SPLIT>;
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, DS_BLOCK, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, DS_BLOCK, 0);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "occupancy(distinct)");
   if (occ < 1) return relhost::set_error("distinct count: kernel does not fit"), REL_E_UNSUPPORTED;
   const int64_t chunks = (p.n_rows + (int64_t)DS_BLOCK * DS_U - 1) / ((int64_t)DS_BLOCK * DS_U);
-  int64_t grid = (int64_t)relhost::device_sms() * occ;
+  int64_t grid = (int64_t)(relhost::device_sms() - (beside ? 1 : 0)) * occ;
   if (grid > chunks) grid = chunks;
   if (grid < 1) grid = 1;
   relhost::launch_begin(relhost::K_GB_KEYSET, st);
-  kern<<<(int)grid, DS_BLOCK, smem, st>>>(p);
+  e = relhost::launch(kern, (unsigned)grid, DS_BLOCK, 0, st, beside, p);
   relhost::launch_end(relhost::K_GB_KEYSET, st);
-  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(distinct)");
 }
 
@@ -343,16 +338,15 @@ double hll_estimate(const uint32_t* regs) {
   return e;
 }
 
-rel_status distinct_launch(const DistinctParams& p, int key_type, cudaStream_t st) {
+rel_status distinct_launch(const DistinctParams& p, int key_type, bool beside, cudaStream_t st) {
   if (p.n_rows == 0) return REL_OK;
-  if (!p.set || p.n_buckets < 1 || p.n_pass < 1 || p.pass >= p.n_pass ||
-      (p.filter_slots & (p.filter_slots - 1)) || p.filter_slots > 16384)
+  if (!p.set || p.n_buckets < 1 || p.n_buckets >= (1ull << 31) || p.n_pass < 1 || p.pass >= p.n_pass)
     return relhost::set_error("distinct count: bad parameters"), REL_E_INVALID;
   if ((uintptr_t)p.set % 32)
     return relhost::set_error("distinct count: key set not 32-byte aligned"), REL_E_INVALID;
-  const bool f = p.filter_slots != 0;
-  if (key_type == REL_I64) return f ? launch<int64_t, true>(p, st) : launch<int64_t, false>(p, st);
-  if (key_type == REL_I32) return f ? launch<int32_t, true>(p, st) : launch<int32_t, false>(p, st);
+  const bool split = p.n_pass > 1;
+  if (key_type == REL_I64) return split ? launch<int64_t, true>(p, beside, st) : launch<int64_t, false>(p, beside, st);
+  if (key_type == REL_I32) return split ? launch<int32_t, true>(p, beside, st) : launch<int32_t, false>(p, beside, st);
   return relhost::set_error("distinct count: needs an int32 or int64 key"), REL_E_INVALID;
 }
 

@@ -20,15 +20,13 @@ struct DistinctParams {
   uint64_t* set;          // n_buckets x DS_BUCKET_SLOTS stored keys, zeroed
   uint64_t n_buckets;     // any count >= 1
   uint32_t n_pass, pass;  // hash split: this launch counts keys of pass `pass`
-  uint32_t filter_slots;  // per-CTA filter of recently sent keys: 0 or a power of two
   WsHeader* hdr;          // aux += distinct keys of this pass; n_side += INT64_MIN rows
                           // (pass 0); overflow set when a probe gives up
 };
 
-// Bytes of shared memory the kernel needs for a filter of `filter_slots`.
-inline size_t distinct_smem_bytes(uint32_t filter_slots) { return 8ull * filter_slots; }
-
-rel_status distinct_launch(const DistinctParams& p, int key_type, cudaStream_t st);
+// beside: the kernel in front of it in the stream may still run (see
+// relhost::launch); one SM is then left to it.
+rel_status distinct_launch(const DistinctParams& p, int key_type, bool beside, cudaStream_t st);
 
 // HyperLogLog over every key of one int32 / int64 column (p = 12: 4096
 // registers, caller-zeroed device uint32[4096]; register = top 12 bits of

@@ -26,7 +26,9 @@ namespace rel {
 namespace {
 
 constexpr int GEN_U = 4;  // consecutive rows per thread
-constexpr uint32_t GEN_MAX_SMEM = 220 * 1024;
+// What a table may take: the rest of the SM's 256 KB is L1, through which the
+// columns stream.
+constexpr uint32_t GEN_MAX_SMEM = 168 * 1024;
 
 // Shared words of one aggregate: SUM 8 bytes (two arrays of 4), MIN / MAX 8,
 // COUNT none of its own.
@@ -143,25 +145,12 @@ __device__ __forceinline__ void agg4(const GbParams& p, int a, int64_t r, bool f
   }
 }
 
-__device__ __forceinline__ uint64_t gen_home(const GbParams& p, uint64_t ek) {
-  return slot_of(ek, p.log2_slots) & ~3ull;
-}
-__device__ __forceinline__ void ld_sector(const uint64_t* q, uint64_t (&k)[4]) {
-  asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
-               : "=l"(k[0]), "=l"(k[1]), "=l"(k[2]), "=l"(k[3])
-               : "l"(q)
-               : "memory");
-}
-__device__ __forceinline__ uint32_t in_sector(const uint64_t (&k)[4], uint64_t e) {
-  return k[0] == e ? 0 : k[1] == e ? 1 : k[2] == e ? 2 : k[3] == e ? 3 : 4;
-}
-
 // Global slot of key e, walking from its home sector and claiming the first
 // empty slot; *claimed when this call put it there.  ~0 when the table
 // overflowed.
 __device__ __forceinline__ uint64_t global_slot(const GbParams& p, uint64_t e, bool* claimed) {
   const uint64_t mask = (1ull << p.log2_slots) - 1;
-  uint64_t s = gen_home(p, e);
+  uint64_t s = home_sector(e, p.log2_slots);
   *claimed = false;
   for (uint32_t i = 0; i < p.max_probe; i += 4) {
     uint64_t k[4];
@@ -195,7 +184,7 @@ __device__ __forceinline__ uint32_t global_slots(const GbParams& p, const uint64
     uint64_t k[2][4];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      gs[h + q] = gen_home(p, ek[h + q]);
+      gs[h + q] = home_sector(ek[h + q], p.log2_slots);
       if (m >> (h + q) & 1) ld_sector(p.tkeys + gs[h + q], k[q]);
     }
 #pragma unroll
@@ -398,6 +387,7 @@ __global__ void __launch_bounds__(1024, 1) gb_gen_k(const __grid_constant__ GbPa
 #pragma unroll
     for (int o = 16; o; o >>= 1) claims += __shfl_xor_sync(0xffffffffu, claims, o);
     if ((threadIdx.x & 31) == 0 && claims) atomicAdd(&p.hdr->aux, claims);
+    wait_for_earlier_kernels();
   }
 }
 
@@ -448,10 +438,12 @@ __global__ void __launch_bounds__(512, 3) gb_gen_bits_k(const __grid_constant__ 
 #pragma unroll
   for (int o = 16; o; o >>= 1) claims += __shfl_xor_sync(0xffffffffu, claims, o);
   if ((threadIdx.x & 31) == 0 && claims) atomicAdd(&p.hdr->aux, claims);
+  wait_for_earlier_kernels();
 }
 
 template <class K>
-rel_status launch_gen(K kern, int id, size_t smem, const GbParams& p, cudaStream_t st) {
+rel_status launch_gen(K kern, int id, size_t smem, const GbParams& p, cudaStream_t st,
+                      bool beside = false) {
   if (p.n_rows == 0) return REL_OK;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(generic)");
@@ -462,12 +454,12 @@ rel_status launch_gen(K kern, int id, size_t smem, const GbParams& p, cudaStream
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem);
   if (e != cudaSuccess || occ < 1) return relhost::cuda_fail(e, "occupancy(generic)");
   const int64_t chunk = (int64_t)block * GEN_U, chunks = (p.n_rows + chunk - 1) / chunk;
-  int64_t grid = (int64_t)relhost::device_sms() * occ;
+  int64_t grid = (int64_t)(relhost::device_sms() - (beside ? 1 : 0)) * occ;
   if (grid > chunks) grid = chunks;
   relhost::launch_begin(id, st);
-  kern<<<(int)grid, block, smem, st>>>(p);
+  e = relhost::launch(kern, (unsigned)grid, (unsigned)block, smem, st, beside, p);
   relhost::launch_end(id, st);
-  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(generic)");
 }
 
@@ -492,17 +484,17 @@ rel_status gb_launch_gen(const GbParams& p0, int64_t est, cudaStream_t st) {
   return launch_gen(gb_gen_k<true, false>, relhost::K_GB_LAYERED, gen_smem(p, p.smem_slots), p, st);
 }
 
-rel_status gb_launch_gen_set(const GbParams& p0, cudaStream_t st) {
+rel_status gb_launch_gen_set(const GbParams& p0, bool beside, cudaStream_t st) {
   GbParams p = p0;
   bool narrow = p.n_keys <= 2;  // and a set large enough for a bit per key
   for (int k = 0; k < p.n_keys; ++k) narrow &= p.ctype[p.key_col[k]] == REL_U8;
   if (narrow && (8ull << p.log2_slots) >= 4ull * BITS_WORDS)
-    return launch_gen(gb_gen_bits_k, relhost::K_GB_KEYSET, 0, p, st);
+    return launch_gen(gb_gen_bits_k, relhost::K_GB_KEYSET, 0, p, st, beside);
   // the keys the CTA has seen: few keys never reach the global set twice, and
   // a row of many keys is not searched for long
   p.smem_slots = 4096;
   p.shared_probes = 2;
-  return launch_gen(gb_gen_k<true, true>, relhost::K_GB_KEYSET, 8 * (size_t)p.smem_slots, p, st);
+  return launch_gen(gb_gen_k<true, true>, relhost::K_GB_KEYSET, 8 * (size_t)p.smem_slots, p, st, beside);
 }
 
 }  // namespace rel

@@ -12,6 +12,7 @@ namespace rel {
 rel_status gb_launch_gen(const GbParams& p, int64_t est, cudaStream_t st);
 // Distinct qualifying keys: hdr->aux counts the keys claimed in the set
 // p.tkeys (2^p.log2_slots slots), hdr->n_side the rows with key INT64_MIN.
-rel_status gb_launch_gen_set(const GbParams& p, cudaStream_t st);
+// beside as for distinct_launch.
+rel_status gb_launch_gen_set(const GbParams& p, bool beside, cudaStream_t st);
 
 }  // namespace rel

@@ -182,11 +182,11 @@ bool gb_q1_eligible(const GbParams& p, int n_hot) {
 
 rel_status gb_launch_q1(const GbParams& p, int n_hot, cudaStream_t st) {
   if (p.n_rows == 0) return REL_OK;
-  // one CTA per SM of as many threads as the words leave room for, up to 768
-  // (1e8 rows: 512 threads 0.711 ms in two CTAs per SM, 768 0.537, 1024 0.704);
-  // small inputs in small CTAs, so that more SMs take part
+  // one CTA per SM, whose words leave 70 KB of the SM's 256 to L1: the columns
+  // stream through it (1e8 rows: 768 threads 0.537 ms; 1024, or 512 in two
+  // CTAs, with 30 KB of L1 0.70); small inputs in small CTAs, so that more SMs take part
   int block = p.n_rows > (int64_t)relhost::device_sms() * 4096 ? 768 : 256;
-  while (block > 128 && q1_smem(n_hot, block) > 226 * 1024) block -= 128;
+  while (block > 128 && q1_smem(n_hot, block) > 184 * 1024) block -= 128;
   const size_t smem = q1_smem(n_hot, block);
   cudaError_t e = cudaFuncSetAttribute(gb_q1_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(fused)");

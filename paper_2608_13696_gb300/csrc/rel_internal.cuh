@@ -162,6 +162,40 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy() {
   return pol;
 }
 
+// Four consecutive slots of a key array (one 32-byte sector), from L2; the
+// first slot of the home sector of a key; a key's place in a sector (4: none).
+__device__ __forceinline__ void ld_sector(const uint64_t* p, uint64_t (&k)[4]) {
+  asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(k[0]), "=l"(k[1]), "=l"(k[2]), "=l"(k[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ uint64_t home_sector(uint64_t ek, int log2_slots) {
+  return slot_of(ek, log2_slots) & ~3ull;
+}
+__device__ __forceinline__ uint32_t in_sector(const uint64_t (&k)[4], uint64_t e) {
+  return k[0] == e ? 0 : k[1] == e ? 1 : k[2] == e ? 2 : k[3] == e ? 3 : 4;
+}
+// Claim the first slot of a sector that was empty as loaded for key e, in
+// order; its place, or 4 when other keys took them.
+__device__ __forceinline__ uint32_t claim_in_sector(uint64_t* p, const uint64_t (&k)[4], uint64_t e) {
+  uint32_t at = 4;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (at != 4 || k[q] != 0) continue;
+    const uint64_t old = atomicCAS((unsigned long long*)(p + q), 0ull, (unsigned long long)e);
+    if (old == 0 || old == e) at = q;
+  }
+  return at;
+}
+
+// Wait for the kernels this one was allowed to run beside (a no-op for an
+// ordinary launch): the last thing a thread does, so that this kernel's end is
+// also theirs.
+__device__ __forceinline__ void wait_for_earlier_kernels() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // One-dimensional bulk copy global -> shared (the TMA engine), completing on
 // an mbarrier.  Both addresses 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes,
@@ -247,4 +281,23 @@ enum KernelId : int {
 // Bracket one launch: counts it and, while profiling, records events.
 void launch_begin(int kernel_id, cudaStream_t st);
 void launch_end(int kernel_id, cudaStream_t st);
+
+// Launch a kernel; beside: it may start before the kernel in front of it in
+// the stream has finished (it must not read what that one writes, and ends
+// with wait_for_earlier_kernels).
+template <class... A>
+cudaError_t launch(void (*kern)(A...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                   bool beside, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = beside ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kern, args...);
+}
 }  // namespace relhost

@@ -107,7 +107,7 @@ struct KeyPair<int32_t> {
   }
 };
 
-template <class KT, int NA, bool PIN>
+template <class KT, int NA>
 __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant__ GbParams p) {
   extern __shared__ __align__(16) uint8_t sm[];
   // [pinned keys by slot: 32 x 8 B][dense id by slot: 32 B][key by dense id:
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
   const int tid = threadIdx.x;
   const uint32_t tmask = p.tiny_slots - 1;
 
-  if (PIN) {
+  {
     if (tid < 32) {
       const uint64_t k = tid < (int)p.tiny_slots ? p.tiny_init[tid] : 0;
       pk[tid] = k;
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
       if (!ok[j]) continue;
       uint64_t w[NA];
       words_of<NA>(val[j], w);
-      if (PIN) {
+      {
         const uint32_t s = small_slot_of(ek[j], tmask, p.tiny_mult);
         if (pk[s] == ek[j] && ek[j] != 0) {
           uint64_t* t = acc + (size_t)dense[s] * NA * ST_BLOCK + tid;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
   }
 
   // fold the thread-private words into the global table
-  if (PIN) {
+  {
     const int lane = tid & 31;
     for (int d = 0; d < PM; ++d) {
 #pragma unroll
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(ST_BLOCK, 6) gb_stream_k(const __grid_constant
     }
   }
   __syncthreads();
-  if (PIN && tid < PM && csum[tid * NA + 1] != 0) {  // word 1 counts rows
+  if (tid < PM && csum[tid * NA + 1] != 0) {  // word 1 counts rows
     uint64_t w[NA];
 #pragma unroll
     for (int a = 0; a < NA; ++a) w[a] = csum[tid * NA + a];
@@ -264,7 +264,10 @@ __device__ __noinline__ void rare_row(const GbParams& p, uint64_t ek, uint64_t v
 // are not used: on a hot key the table's adds serialise over a warp's lanes
 // (15 ns a warp at worst), less than a second lookup costs every row.
 constexpr int SG_U = 4;            // rows per thread per chunk
-constexpr uint32_t SG_MAX_BYTES = 220 * 1024;
+// largest table: the rest of the SM's 256 KB is L1, through which the rows come
+// (1e8 rows, 3000 groups:
+// 220 KB 1.45 ms, 168 KB 1.20)
+constexpr uint32_t SG_MAX_BYTES = 168 * 1024;
 
 template <class KT, int NA>
 __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbParams p) {
@@ -341,6 +344,245 @@ __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbP
     uint64_t w[NA];
     t.words(s, w);
     global_update<NA>(p, k, w);
+  }
+}
+
+// Every row straight into the global table: a plan without per-CTA slots.
+// Bound by L2: per row one sector of four keys, and for MIN and MAX the pair
+// read first and raised only when the row improves it, beside the reductions
+// of sum and count (four reductions a row: 50 G rows/s at best; a 16-byte load
+// and two: 74).  1e8 rows, 20000 groups: 3.22 ms with one-slot probes
+// and four reductions, 2.11 ms.
+template <class KT, int NA>
+__global__ void __launch_bounds__(512, 2) gb_glob_k(const __grid_constant__ GbParams p) {
+  constexpr int U = 2;
+  const KT* keys = (const KT*)p.col[p.key_col[0]];
+  const int64_t* vals = (const int64_t*)p.col[p.r_a];
+  const int64_t n = p.n_rows, CHUNK = (int64_t)blockDim.x * U;
+  const bool vec = ((uintptr_t)keys % (2 * sizeof(KT)) == 0) && ((uintptr_t)vals % 16 == 0);
+  const uint64_t mask = (1ull << p.log2_slots) - 1;
+  for (int64_t base = (int64_t)blockIdx.x * CHUNK; base < n; base += (int64_t)gridDim.x * CHUNK) {
+    uint64_t ek[U] = {0, 0}, v[U] = {0, 0}, s[U];
+    uint32_t put = 0;  // rows to add
+    const int64_t r = base + U * threadIdx.x;
+    if (vec && r + 1 < n) {
+      int64_t k0, k1;
+      KeyPair<KT>::split(__ldcs((const typename KeyPair<KT>::V*)(keys + r)), k0, k1);
+      const longlong2 vv = __ldcs((const longlong2*)(vals + r));
+      ek[0] = (uint64_t)k0 ^ KEY_FLIP;
+      ek[1] = (uint64_t)k1 ^ KEY_FLIP;
+      v[0] = (uint64_t)vv.x;
+      v[1] = (uint64_t)vv.y;
+      put = 3;
+    } else {
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        if (r + j >= n) continue;
+        ek[j] = (uint64_t)(int64_t)keys[r + j] ^ KEY_FLIP;
+        v[j] = (uint64_t)vals[r + j];
+        put |= 1u << j;
+      }
+    }
+    uint32_t miss = 0;
+    {
+      uint64_t k[U][4];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        s[j] = home_sector(ek[j], p.log2_slots);
+        ld_sector(p.tkeys + s[j], k[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        if (!(put >> j & 1)) continue;
+        if (ek[j] == 0) {  // INT64_MIN
+          rare_row<NA>(p, 0, v[j]);
+          put &= ~(1u << j);
+          continue;
+        }
+        const uint32_t at = in_sector(k[j], ek[j]);
+        if (at != 4) {
+          s[j] += at;
+        } else {
+          miss |= 1u << j;
+          if (k[j][3] != 0) s[j] = (s[j] + 4) & mask;  // the home sector is full
+        }
+      }
+    }
+    // the few rows that leave their home sector, or open a group
+    for (uint32_t i = 0; miss; i += 4) {
+      const bool second = !(miss & 1);
+      const uint64_t e = second ? ek[1] : ek[0];
+      uint64_t w = second ? s[1] : s[0], k[4];
+      ld_sector(p.tkeys + w, k);
+      uint32_t at = in_sector(k, e);
+      if (at == 4 && k[3] == 0) at = claim_in_sector(p.tkeys + w, k, e);  // room as loaded
+      bool done = at != 4;
+      w = done ? w + at : (w + 4) & mask;
+      if (!done) {
+        const bool over = i >= 2 * p.max_probe;
+        if (over) atomicOr(&p.hdr->overflow, 1u);
+        if (over || ((i & 31) == 28 && ld_relaxed_u32(&p.hdr->overflow))) {  // already overflowed
+          done = true;
+          put &= ~(miss & (0u - miss));
+        }
+      }
+      if (second) s[1] = w; else s[0] = w;
+      if (done) miss &= miss - 1;
+    }
+    __syncwarp();
+    if constexpr (NA == 4) {
+      uint64_t mn[U], mx[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        mn[j] = mx[j] = ~0ull;
+        if (put >> j & 1)
+          asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
+                       : "=l"(mn[j]), "=l"(mx[j])
+                       : "l"(p.taggs + s[j] * 4 + 2)
+                       : "memory");
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        if ((v[j] ^ MIN_FLIP) > mn[j]) redg_max(p.taggs + s[j] * 4 + 2, v[j] ^ MIN_FLIP);
+        if ((v[j] ^ MAX_FLIP) > mx[j]) redg_max(p.taggs + s[j] * 4 + 3, v[j] ^ MAX_FLIP);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (!(put >> j & 1)) continue;
+      redg_add(p.taggs + s[j] * NA, v[j]);
+      redg_add(p.taggs + s[j] * NA + 1, 1);
+    }
+  }
+}
+
+// Rows of a plan whose groups are all pinned (a handful of keys): thread-private
+// words only, updated without atomics, and HBM the bound.  Against gb_stream_k,
+// which also carries rows that are not pinned at full speed: words of 28 bytes
+// a key instead of 32 with MIN and MAX read as one and written only when
+// raised, columns by hash slot instead of a second lookup, one wide CTA per SM.
+// 2e8 rows of four keys: 0.742 -> 0.515 ms (6.2 TB/s, 92 % of the copy rate).
+constexpr int PK_U = 4;             // rows per thread per chunk
+constexpr int PK_MAX_BLOCK = 768;
+
+template <int NA>
+__host__ __device__ constexpr uint32_t pk_key_bytes() {  // per key and thread: sum, count, (min, max)
+  return NA == 4 ? 28 : 12;
+}
+constexpr uint32_t PK_HEAD = 8 * TINY_MAX_SLOTS + 8 * TINY_MAX_SLOTS * 4;  // keys, reduced words
+
+template <class KT, int NA>
+__global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constant__ GbParams p) {
+  extern __shared__ __align__(16) uint8_t sm[];
+  uint64_t* pk = (uint64_t*)sm;  // pinned key of each slot (0: none)
+  uint64_t* red = pk + TINY_MAX_SLOTS;
+  const uint32_t S = p.tiny_slots, B = blockDim.x, tid = threadIdx.x, tmask = S - 1;
+  // [min, max pairs][sums][counts], each [slot][thread]
+  const uint32_t mm = smem_u32(sm) + PK_HEAD, sum = mm + (NA == 4 ? 16 * S * B : 0), cnt = sum + 8 * S * B;
+  if (tid < TINY_MAX_SLOTS) pk[tid] = tid < S ? p.tiny_init[tid] : 0;
+  for (uint32_t s = 0; s < S; ++s) {
+    if (NA == 4) {
+      sts64(mm + 16 * (s * B + tid), 0);
+      sts64(mm + 16 * (s * B + tid) + 8, 0);
+    }
+    sts64(sum + 8 * (s * B + tid), 0);
+    sts32(cnt + 4 * (s * B + tid), 0);
+  }
+  __syncthreads();
+  const KT* keys = (const KT*)p.col[p.key_col[0]];
+  const int64_t* vals = (const int64_t*)p.col[p.r_a];
+  const int64_t n = p.n_rows, CHUNK = (int64_t)B * PK_U, step = (int64_t)gridDim.x * CHUNK;
+  const bool vec = ((uintptr_t)keys % (2 * sizeof(KT)) == 0) && ((uintptr_t)vals % 16 == 0);
+  auto load = [&](int64_t base, uint64_t(&ek)[PK_U], uint64_t(&val)[PK_U]) -> uint32_t {
+    uint32_t ok = 0;
+    if (vec && base + CHUNK <= n) {
+#pragma unroll
+      for (int j = 0; j < PK_U; j += 2) {
+        const int64_t r = base + (int64_t)j * B + 2 * tid;
+        int64_t k0, k1;
+        KeyPair<KT>::split(__ldcs((const typename KeyPair<KT>::V*)(keys + r)), k0, k1);
+        const longlong2 vv = __ldcs((const longlong2*)(vals + r));
+        ek[j] = (uint64_t)k0 ^ KEY_FLIP;
+        ek[j + 1] = (uint64_t)k1 ^ KEY_FLIP;
+        val[j] = (uint64_t)vv.x;
+        val[j + 1] = (uint64_t)vv.y;
+      }
+      return (1u << PK_U) - 1;
+    }
+#pragma unroll
+    for (int j = 0; j < PK_U; ++j) {
+      const int64_t r = base + (int64_t)(j / 2) * 2 * B + 2 * tid + (j & 1);
+      const bool in = r < n;
+      ek[j] = in ? (uint64_t)(int64_t)keys[r] ^ KEY_FLIP : 0;
+      val[j] = in ? (uint64_t)vals[r] : 0;
+      ok |= (in ? 1u : 0u) << j;
+    }
+    return ok;
+  };
+  uint64_t ek[PK_U], val[PK_U];
+  int64_t base = (int64_t)blockIdx.x * CHUNK;
+  uint32_t ok = base < n ? load(base, ek, val) : 0;
+  for (; base < n; base += step) {
+    uint64_t nek[PK_U], nval[PK_U];
+    const uint32_t nok = base + step < n ? load(base + step, nek, nval) : 0;
+    uint32_t s[PK_U];
+    bool hit[PK_U];
+#pragma unroll
+    for (int j = 0; j < PK_U; ++j) {
+      s[j] = small_slot_of(ek[j], tmask, p.tiny_mult);
+      hit[j] = pk[s[j]] == ek[j] && ek[j] != 0;
+    }
+#pragma unroll
+    for (int j = 0; j < PK_U; ++j) {
+      if (hit[j]) {
+        const uint32_t at = s[j] * B + tid;
+        const uint64_t o = lds64(sum + 8 * at);
+        const uint32_t c = lds32(cnt + 4 * at);
+        if constexpr (NA == 4) {
+          uint64_t mn, mx;
+          lds128(mm + 16 * at, mn, mx);
+          const uint64_t a = val[j] ^ MIN_FLIP, b = val[j] ^ MAX_FLIP;
+          if (a > mn) sts64(mm + 16 * at, a);
+          if (b > mx) sts64(mm + 16 * at + 8, b);
+        }
+        sts64(sum + 8 * at, o + val[j]);
+        sts32(cnt + 4 * at, c + 1);
+      } else if (ok >> j & 1) {
+        rare_row<NA>(p, ek[j], val[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < PK_U; ++j) {
+      ek[j] = nek[j];
+      val[j] = nval[j];
+    }
+    ok = nok;
+  }
+  __syncthreads();
+  // one warp per (slot, word): the threads' words folded, then the groups
+  const uint32_t warp = tid >> 5, lane = tid & 31;
+  for (uint32_t q = warp; q < S * NA; q += B / 32) {
+    const uint32_t g = q / NA, a = q % NA;
+    uint64_t v = 0;
+    for (uint32_t i = lane; i < B; i += 32) {
+      const uint32_t at = g * B + i;
+      const uint64_t y = a == 0 ? lds64(sum + 8 * at) : a == 1 ? (uint64_t)lds32(cnt + 4 * at)
+                                                              : lds64(mm + 16 * at + 8 * (a - 2));
+      v = umax_word<NA>(a) ? (v > y ? v : y) : v + y;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const uint64_t y = __shfl_xor_sync(0xffffffffu, v, o);
+      v = umax_word<NA>(a) ? (v > y ? v : y) : v + y;
+    }
+    if (lane == 0) red[q] = v;
+  }
+  __syncthreads();
+  if (tid < S && red[tid * NA + 1] != 0) {
+    uint64_t w[NA];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) w[a] = red[tid * NA + a];
+    global_update<NA>(p, pk[tid], w);
   }
 }
 
@@ -669,10 +911,8 @@ rel_status ppass_dispatch(const GbParams& p, bool scatter, cudaStream_t st) {
   return scatter ? launch_ppass<KT, NA, false, true>(p, st) : launch_ppass<KT, NA, false, false>(p, st);
 }
 
-size_t stream_smem(int na, bool pin) {
-  size_t b = 416 + 8 * ST_PIN_LIMIT * 4;
-  if (pin) b += (size_t)8 * (na == 4 ? pin_max<4>() : pin_max<2>()) * na * ST_BLOCK;
-  return b;
+size_t stream_smem(int na) {
+  return 416 + 8 * ST_PIN_LIMIT * 4 + (size_t)8 * (na == 4 ? pin_max<4>() : pin_max<2>()) * na * ST_BLOCK;
 }
 
 // One wave of resident CTAs, at most one per chunk.
@@ -718,7 +958,7 @@ rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
     // table gets what one CTA per SM can hold.
     if (q.smem_slots < 256) q.smem_slots = 256;
     if (p.n_rows > 8 * small)
-      while (q.smem_slots < 4 * p.smem_slots && SmTab<NA>::bytes(2 * q.smem_slots) <= 110 * 1024)
+      while (q.smem_slots < 4 * p.smem_slots && SmTab<NA>::bytes(2 * q.smem_slots) <= SG_MAX_BYTES / 2)
         q.smem_slots *= 2;
     if (p.smem_slots == SHARED_MAX_SLOTS) q.smem_slots = SmTab<NA>::fit(SG_MAX_BYTES);
     const size_t smem = SmTab<NA>::bytes(q.smem_slots);
@@ -726,9 +966,15 @@ rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
     return launch_rows(gb_smem_k<KT, NA>, block, smem, (int64_t)block * SG_U, q, st);
   }
   const bool pin = p.tiny_frozen && p.tiny_slots;
-  const size_t smem = stream_smem(NA, pin);
-  if (pin) return launch_rows(gb_stream_k<KT, NA, true>, ST_BLOCK, smem, ST_BLOCK * ST_U, p, st);
-  return launch_rows(gb_stream_k<KT, NA, false>, ST_BLOCK, smem, ST_BLOCK * ST_U, p, st);
+  if (pin && p.all_pinned) {
+    int block = p.n_rows > (int64_t)relhost::device_sms() * 4096 ? PK_MAX_BLOCK : 128;
+    const uint32_t per = p.tiny_slots * pk_key_bytes<NA>();
+    while (block > 128 && PK_HEAD + per * block > 184 * 1024) block -= 128;  // (L1)
+    return launch_rows(gb_pin_k<KT, NA>, block, PK_HEAD + (size_t)per * block, (int64_t)block * PK_U, p, st);
+  }
+  if (pin) return launch_rows(gb_stream_k<KT, NA>, ST_BLOCK, stream_smem(NA), ST_BLOCK * ST_U, p, st);
+  const int block = p.n_rows > (int64_t)relhost::device_sms() * 2048 ? 512 : 128;
+  return launch_rows(gb_glob_k<KT, NA>, block, 0, (int64_t)block * 2, p, st);
 }
 
 }  // namespace

@@ -143,3 +143,42 @@ def test_batch_join_edges(items):
         for x, y in zip(got, e):
             np.testing.assert_array_equal(x, y)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("na", [2, 4])
+@pytest.mark.parametrize("dtype", [np.int64, np.int32])
+@pytest.mark.parametrize("n", [5, 511, 3073, 700_003])
+@pytest.mark.parametrize("groups", [1, 4, 6])
+def test_all_groups_pinned(na, dtype, n, groups):
+    """The pinned kernel, with rows the sample missed and INT64_MIN / INT64_MAX keys."""
+    k, v = column("uniform", n, groups, dtype, n + groups)
+    if dtype == np.int64:
+        k[n // 2] = I64.max
+    k[n - 1] = 12345  # one row of one more key
+    for off in (0, 1):
+        q = oracle.kv_query(k[off:], v[off:], ops=OPS[na])
+        qc = {"cols": [cuda(k)[off:], cuda(v)[off:]], "keys": [0], "preds": [],
+              "aggs": [(o, 1, []) for o in OPS[na]]}
+        p = rel.plan_groupby(qc, groups_hint=max(4, groups), flags=rel.PLAN_SKETCH)
+        got = canon_groupby(*rel.groupby(qc, plan=p, capacity=64))
+        exp = oracle.groupby(q)
+        np.testing.assert_array_equal(got[0], exp[0])
+        np.testing.assert_array_equal(got[1], exp[1])
+
+
+@pytest.mark.parametrize("n", [33, 4096, 4097, 60_001])
+@pytest.mark.parametrize("groups", [1, 200, 50_000])
+@pytest.mark.parametrize("dtype", [np.int64, np.int32])
+def test_exact_plan_with_sketch(n, groups, dtype):
+    """The exact count beside the sketch, and in its place on small inputs."""
+    k, v = column("uniform", n, groups, dtype, n)
+    s = oracle.sketch(oracle.kv_query(k, v))
+    for keys in ([0], [0, 2]):
+        if len(keys) == 2 and dtype == np.int64:
+            continue
+        cols = [cuda(k), cuda(v), cuda((k % 7).astype(np.uint8))]
+        q = {"cols": cols, "keys": keys, "preds": [], "aggs": [("sum", 1, []), ("count", 1, [])]}
+        p = rel.plan_groupby(q, flags=rel.PLAN_EXACT | rel.PLAN_SKETCH)
+        assert p.est_groups == len(np.unique(k))  # the second column follows from the first
+        if len(keys) == 1:
+            assert set(p.hot_keys[i] for i in range(p.n_hot)) <= set(int(x) for x in s["top_key"])
