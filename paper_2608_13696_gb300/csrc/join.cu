@@ -10,10 +10,10 @@
 // enough to stay in the GB300's L2 (whose random-access sweet spot is below
 // ~64 MB) while the probe keys stream from HBM with evict-first loads and the
 // outputs leave with streaming stores.  The payload gather is fused into the
-// probe.  Every probe row's first slot is loaded before any is resolved,
-// probe keys arrive in 16-byte vector loads, and each warp compacts its
-// lanes' matches with a ballot / popc and reserves output space with one
-// atomic.
+// probe.  Slots come in pairs that fill one 32-byte sector: a key's sequence
+// starts at its home pair and one 256-bit load shows both slots, so ten of
+// eleven unique keys (load 0.48) are decided by their first load; the others
+// are finished in one loop per four rows, each lane on its own next row.
 #include "join.cuh"
 
 namespace rel {
@@ -22,20 +22,27 @@ namespace {
 
 constexpr int J_BLOCK = 256;
 
-// One slot (key, build row index), marked evict-last in L2 so that the table
-// outlives the streamed probe keys (evict-first) and the streamed outputs.
-__device__ __forceinline__ void ld_slot(const JoinSlot* p, uint64_t& ek, int32_t& bidx) {
-  unsigned long long a, b;
-  asm volatile(
-      "{\n\t.reg .b64 pol;\n\t"
-      "createpolicy.fractional.L2::evict_last.b64 pol, 1.0;\n\t"
-      "ld.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], pol;\n\t}"
-      : "=l"(a), "=l"(b)
-      : "l"(p));
-  ek = a;
-  bidx = (int32_t)(uint32_t)b;
+// A pair of slots: keys a and b, build rows x and y.  Marked evict-last in L2
+// so that the table outlives the streamed probe keys (evict-first) and the
+// streamed outputs.
+struct Pair {
+  uint64_t a, b;
+  int32_t x, y;
+};
+__device__ __forceinline__ Pair ld_pair(const JoinSlot* p, uint64_t pol) {
+  unsigned long long k0, v0, k1, v1;
+  asm volatile("ld.global.L2::cache_hint.v4.u64 {%0, %1, %2, %3}, [%4], %5;"
+               : "=l"(k0), "=l"(v0), "=l"(k1), "=l"(v1)
+               : "l"(p), "l"(pol));
+  return Pair{k0, k1, (int32_t)(uint32_t)v0, (int32_t)(uint32_t)v1};
+}
+__device__ __forceinline__ uint64_t home_pair(uint64_t ek, int log2_slots) {
+  return slot_of(ek, log2_slots) & ~1ull;
 }
 
+// Every build row claims the first empty slot from its home pair on; the first
+// is tried without a look (the table is at most half full).  10^6 rows: 48 us,
+// as before, bound by the latency of the claims.
 __global__ void __launch_bounds__(J_BLOCK) join_build_k(const __grid_constant__ JoinParams p,
                                                         const int64_t* __restrict__ keys,
                                                         const int64_t* __restrict__ payload,
@@ -44,198 +51,205 @@ __global__ void __launch_bounds__(J_BLOCK) join_build_k(const __grid_constant__ 
   bool dup = false;
   for (int64_t j = (int64_t)blockIdx.x * J_BLOCK + threadIdx.x; j < n;
        j += (int64_t)gridDim.x * J_BLOCK) {
-    const uint64_t ek = (uint64_t)__ldg((const long long*)keys + j) ^ KEY_FLIP;
-    const long long pay = __ldg((const long long*)payload + j);
+    const uint64_t ek = (uint64_t)__ldcs((const long long*)keys + j) ^ KEY_FLIP;
+    const long long pay = __ldcs((const long long*)payload + j);
     p.pay[j] = pay;  // the table's copy of the payload column
-    if (ek == 0) {  // INT64_MIN: side list
-      const unsigned long long pos = atomicAdd(&p.hdr->n_side, 1ull);
-      p.side[pos] = JoinVal{pay, (int32_t)j, 0};
+    if (ek == 0) {   // INT64_MIN: side list
+      p.side[atomicAdd(&p.hdr->n_side, 1ull)] = JoinVal{pay, (int32_t)j, 0};
       continue;
     }
-    uint64_t s = slot_of(ek, p.log2_slots);
-    bool placed = false;
-    for (uint64_t i = 0; i <= mask; ++i) {
-      uint64_t cur = ld_relaxed((const uint64_t*)&p.slots[s].ek);
-      if (cur == 0) {
-        cur = atomicCAS(&p.slots[s].ek, 0ull, (unsigned long long)ek);
-        if (cur == 0) {
-          p.slots[s].bidx = (int32_t)j;
-          placed = true;
-          break;
-        }
-      }
-      // Two inserts of one key start at the same slot and claim slots in
-      // probe order, so the later one always passes the earlier one's slot:
-      // duplicates are always noticed.
-      if (cur == ek) dup = true;
+    uint64_t s = home_pair(ek, p.log2_slots);
+    unsigned long long cur = atomicCAS(&p.slots[s].ek, 0ull, (unsigned long long)ek);
+    // Two inserts of one key start at the same slot and claim slots in probe
+    // order, so the later one always passes the earlier one's slot:
+    // duplicates are always noticed.
+    for (uint64_t i = 0; cur != 0 && i < mask; ++i) {
+      dup |= cur == ek;
       s = (s + 1) & mask;
+      cur = ld_relaxed((const uint64_t*)&p.slots[s].ek);
+      if (cur == 0) cur = atomicCAS(&p.slots[s].ek, 0ull, (unsigned long long)ek);
     }
-    if (!placed) atomicOr(&p.hdr->overflow, 1u);
+    if (cur == 0)
+      p.slots[s].bidx = (int32_t)j;
+    else
+      atomicOr(&p.hdr->overflow, 1u);
   }
   if (dup) atomicOr(&p.hdr->dups, 1u);
 }
 
-// Next match of a lane's probe sequence.  State: slot s (table) or index s
-// into the side list (key INT64_MIN).  Returns false when the sequence ends.
-__device__ __forceinline__ bool next_match(const JoinParams& p, uint64_t ek, bool side,
-                                           uint64_t n_side, uint64_t& s, int64_t& pay,
-                                           int32_t& bidx) {
-  if (side) {
-    if (s >= n_side) return false;
-    const JoinVal v = p.side[s++];
-    pay = v.payload;
-    bidx = v.bidx;
-    return true;
-  }
-  const uint64_t mask = (1ull << p.log2_slots) - 1;
-  for (uint64_t i = 0; i <= mask; ++i) {
-    uint64_t k;
-    ld_slot(p.slots + s, k, bidx);
-    if (k == 0) return false;
-    s = (s + 1) & mask;
-    if (k == ek) {
-      pay = p.pay[bidx];
-      return true;
-    }
-  }
-  return false;
-}
+constexpr int J_FLUSH = 256;             // matches of a warp that are written at once
+constexpr int J_BUF = J_FLUSH + 32 * 4;  // ... and room for one more round
+constexpr int J_CTAS = 4;
 
-// Probe with J_IT rows per thread in flight, in groups of J_G: every row of
-// a group has its first slot (key, payload, build index) loaded before any is
-// resolved, so a warp keeps J_G independent L2 round trips outstanding per
-// lane.  With unique build keys (no duplicate seen while building) a row
-// stops at its first match; otherwise -- and for the INT64_MIN side list --
-// it walks its whole probe sequence.  Matches are written in row-slot order:
-// one atomic per warp and group reserves the output, each row-slot's matches
-// are compacted with a ballot, so consecutive lanes write consecutive
-// entries.  Rows: base + v * 2 * J_BLOCK + 2 * tid + {0, 1}, probe keys read
-// two at a time with 16-byte loads.
-constexpr int J_IT = 8;
-constexpr int J_G = 4;
-
-template <bool EMIT>
-__global__ void __launch_bounds__(J_BLOCK) join_probe_fast_k(const __grid_constant__ JoinParams p,
-                                                             const __grid_constant__ JoinOut o,
-                                                             const int64_t* __restrict__ probe,
-                                                             int64_t n) {
+// Probe U rows per thread.
+//  * Unique build keys (no duplicate seen while building): a row is done at its
+//    first match, all of them in one round.
+//  * Otherwise a row's sequence is walked to its first empty slot, all U rows a
+//    pair further per round.
+//  * Rows with key INT64_MIN walk the side list.
+// A warp collects its matches (probe row, build row) in shared memory and, from
+// J_FLUSH on, reserves the output with one atomic -- all warps take them from
+// one address, which serves 1.6 G/s: one per 128 rows was 78 us of a 16e6-row
+// probe -- gathers the payloads and writes all three columns densely.
+// 16e6 rows into 10^6 keys, 90 % found: 241 -> 202 us, counting 156 -> 124;
+// 400 009 rows into 60 013 keys three times each: 119 -> 41, counting 102 -> 24.
+// Bound by instruction issue (half of the slots) and by the lookups that go on
+// past the home pair, which hold up their warps.
+template <bool EMIT, int U>
+__global__ void __launch_bounds__(J_BLOCK, J_CTAS) join_probe_k(const __grid_constant__ JoinParams p,
+                                                                const __grid_constant__ JoinOut o,
+                                                                const int64_t* __restrict__ probe,
+                                                                int64_t n) {
+  __shared__ int2 bufs[EMIT ? J_BLOCK / 32 : 1][EMIT ? J_BUF : 1];
+  int2* buf = bufs[EMIT ? threadIdx.x / 32 : 0];
+  unsigned fill = 0;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const uint64_t mask = (1ull << p.log2_slots) - 1;
   const bool unique = ld_relaxed_u32(&p.hdr->dups) == 0;
-  const uint64_t n_side = p.hdr->n_side;
+  const uint64_t n_side = p.hdr->n_side, cap = (uint64_t)o.capacity;
+  const uint64_t pol = l2_evict_last_policy();
   const bool vec = (uintptr_t)probe % 16 == 0;
   unsigned long long counted = 0;
-  const int64_t tile = (int64_t)J_BLOCK * J_IT;
-  for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
-    uint64_t ek[J_IT];
-    int64_t row[J_IT];
+  constexpr int64_t TILE = (int64_t)J_BLOCK * U;
+  // row of slot j
+  auto row = [&](int64_t base, int j) -> int64_t {
+    return U == 1 ? base + threadIdx.x : base + (j / 2) * 2 * J_BLOCK + 2 * threadIdx.x + (j & 1);
+  };
+  auto push = [&](bool h, int64_t r, int32_t b) {
+    const unsigned v = __ballot_sync(0xffffffffu, h);
+    if (h) buf[fill + __popc(v & lt)] = make_int2((int32_t)r, b);
+    fill += __popc(v);
+  };
+  auto flush = [&]() {  // the warp converged; streaming stores keep the table in L2
+    __syncwarp();
+    unsigned long long wb = 0;
+    if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)fill);
+    wb = __shfl_sync(0xffffffffu, wb, 0);
+    const unsigned room = wb >= cap ? 0 : cap - wb < fill ? (unsigned)(cap - wb) : fill;
+    for (unsigned i = lane; i < room; i += 32 * 2) {
+      int2 e[2];
+      long long pay[2];
 #pragma unroll
-    for (int v = 0; v < J_IT / 2; ++v) {
-      const int64_t r = base + (int64_t)v * 2 * J_BLOCK + 2 * threadIdx.x;
-      row[2 * v] = r;
-      row[2 * v + 1] = r + 1;
-      if (vec && r + 1 < n) {
-        const longlong2 kk = __ldcs((const longlong2*)(probe + r));
-        ek[2 * v] = (uint64_t)kk.x ^ KEY_FLIP;
-        ek[2 * v + 1] = (uint64_t)kk.y ^ KEY_FLIP;
-      } else {
-        ek[2 * v] = r < n ? (uint64_t)__ldcs((const long long*)probe + r) ^ KEY_FLIP : 0;
-        ek[2 * v + 1] = r + 1 < n ? (uint64_t)__ldcs((const long long*)probe + r + 1) ^ KEY_FLIP : 0;
+      for (int q = 0; q < 2; ++q)
+        if (i + 32 * q < room) {
+          e[q] = buf[i + 32 * q];
+          pay[q] = __ldg(p.pay + e[q].y);
+        }
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        if (i + 32 * q < room) {
+          __stcs(o.probe_idx + wb + i + 32 * q, e[q].x);
+          __stcs(o.build_idx + wb + i + 32 * q, e[q].y);
+          __stcs((long long*)o.payload + wb + i + 32 * q, pay[q]);
+        }
+    }
+    fill = 0;
+    __syncwarp();
+  };
+  for (int64_t base = (int64_t)blockIdx.x * TILE; base < n; base += (int64_t)gridDim.x * TILE) {
+    uint64_t ek[U], s[U];
+    uint32_t side = 0;
+    if (U > 1 && vec && base + TILE <= n) {
+#pragma unroll
+      for (int j = 0; j < U; j += 2) {
+        const longlong2 kk = __ldcs((const longlong2*)(probe + row(base, j)));
+        ek[j] = (uint64_t)kk.x ^ KEY_FLIP;
+        ek[j + (U > 1)] = (uint64_t)kk.y ^ KEY_FLIP;
+      }
+#pragma unroll
+      for (int j = 0; j < U; ++j) side |= (ek[j] == 0 ? 1u : 0u) << j;
+    } else {
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const bool in = row(base, j) < n;
+        ek[j] = in ? (uint64_t)__ldcs((const long long*)probe + row(base, j)) ^ KEY_FLIP : 0;
+        side |= (in && ek[j] == 0 ? 1u : 0u) << j;
       }
     }
+    uint32_t live = 0;
 #pragma unroll
-    for (int g = 0; g < J_IT; g += J_G) {
-      uint64_t s[J_G], k[J_G];
-      int64_t pay[J_G];
-      int32_t bidx[J_G];
-      bool hit[J_G], slow[J_G];
+    for (int j = 0; j < U; ++j) {
+      s[j] = home_pair(ek[j], p.log2_slots);
+      live |= (ek[j] != 0 ? 1u : 0u) << j;
+    }
+    uint64_t walked = 0;
+    do {
+      Pair q[U];
+      uint32_t m = 0;  // bit j: slot a of row j matches; bit 8 + j: slot b
 #pragma unroll
-      for (int q = 0; q < J_G; ++q) {
-        const bool valid = row[g + q] < n;
-        slow[q] = valid && (ek[g + q] == 0 || !unique);
-        s[q] = slot_of(ek[g + q], p.log2_slots);
-        k[q] = 0;
-        if (valid && !slow[q]) ld_slot(p.slots + s[q], k[q], bidx[q]);
+      for (int j = 0; j < U; ++j)
+        if (unique || (live >> j & 1)) q[j] = ld_pair(p.slots + s[j], pol);
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        if (!(live >> j & 1)) continue;
+        m |= (q[j].a == ek[j] ? 1u : 0u) << j | (q[j].b == ek[j] ? 256u : 0u) << j;
+        if (q[j].b == 0) live ^= 1u << j;  // an empty slot ends the sequence
+        s[j] = (s[j] + 2) & mask;
       }
+      if (unique) {
+        live &= ~(m | m >> 8);
+        // what the first pair did not decide: each lane on its own next row
+        for (uint64_t i = 0; live && i <= U * mask; i += 2) {
+          const uint32_t bit = live & (0u - live);
+          uint64_t k = 0, w = 0;
 #pragma unroll
-      for (int q = 0; q < J_G; ++q) {
-        hit[q] = false;
-        if (row[g + q] < n && !slow[q]) {
-          for (uint64_t step = 0; step <= mask && k[q] != 0 && k[q] != ek[g + q]; ++step) {
-            s[q] = (s[q] + 1) & mask;
-            ld_slot(p.slots + s[q], k[q], bidx[q]);
-          }
-          hit[q] = k[q] == ek[g + q];
-        }
-      }
-      // the payload gather of every hit of the group
-#pragma unroll
-      for (int q = 0; q < J_G; ++q)
-        if (EMIT && hit[q]) pay[q] = __ldg(p.pay + bidx[q]);
-      unsigned m[J_G];
-      unsigned total = 0;
-#pragma unroll
-      for (int q = 0; q < J_G; ++q) {
-        m[q] = __ballot_sync(0xffffffffu, hit[q]);
-        total += __popc(m[q]);
-      }
-      if (!EMIT) {
-        counted += lane == 0 ? total : 0;
-      } else if (total) {
-        unsigned long long wb = 0;
-        if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)total);
-        wb = __shfl_sync(0xffffffffu, wb, 0);
-#pragma unroll
-        for (int q = 0; q < J_G; ++q) {
-          if (hit[q]) {
-            const uint64_t pos = wb + __popc(m[q] & lt);
-            if (pos < (uint64_t)o.capacity) {  // streaming stores: keep the table in L2
-              __stcs(o.probe_idx + pos, (int32_t)row[g + q]);
-              __stcs(o.build_idx + pos, bidx[q]);
-              __stcs((long long*)o.payload + pos, (long long)pay[q]);
+          for (int j = 0; j < U; ++j)
+            if (bit == 1u << j) {
+              k = ek[j];
+              w = s[j];
             }
-          }
-          wb += __popc(m[q]);
-        }
-      }
-      // rows that may match more than once (or the INT64_MIN side list): walk
-      // the whole sequence, one match per round, compacted per round
+          const Pair r = ld_pair(p.slots + w, pol);
+          const bool e0 = r.a == k, e1 = r.b == k;
 #pragma unroll
-      for (int q = 0; q < J_G; ++q) {
-        if (!__any_sync(0xffffffffu, slow[q])) continue;
-        const bool side = ek[g + q] == 0;
-        uint64_t qs = side ? 0 : slot_of(ek[g + q], p.log2_slots);
-        bool active = slow[q];
-        while (__any_sync(0xffffffffu, active)) {
-          int64_t wp = 0;
-          int32_t wi = 0;
-          bool h = false;
-          if (active) {
-            h = next_match(p, ek[g + q], side, n_side, qs, wp, wi);
-            active = h;
-          }
-          if (!EMIT) {
-            counted += h;
-            continue;
-          }
-          const unsigned mm = __ballot_sync(0xffffffffu, h);
-          if (!mm) continue;
+          for (int j = 0; j < U; ++j)
+            if (bit == 1u << j) {
+              s[j] = (w + 2) & mask;
+              q[j].x = r.x;
+              q[j].y = r.y;
+            }
+          m |= (e0 ? bit : 0u) | (e1 ? bit << 8 : 0u);
+          if (e0 || e1 || r.b == 0) live ^= bit;
+        }
+        __syncwarp();
+      }
+      if (EMIT) {
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const bool x = m >> j & 1, y = m >> (8 + j) & 1;
+          push(x || (unique && y), row(base, j), x ? q[j].x : q[j].y);
+          if (!unique) push(y, row(base, j), q[j].y);
+        }
+        if (fill >= J_FLUSH) flush();
+      } else {
+        counted += __popc(m);
+      }
+    } while (__any_sync(0xffffffffu, live != 0) && (walked += 2) <= mask);
+    // INT64_MIN rows: every build row of the side list
+    if (__any_sync(0xffffffffu, side != 0)) {
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        const unsigned m = __ballot_sync(0xffffffffu, side >> j & 1);
+        if (!m) continue;
+        if (!EMIT) {
+          counted += side >> j & 1 ? n_side : 0;
+          continue;
+        }
+        for (uint64_t i = 0; i < n_side; ++i) {
           unsigned long long wb = 0;
-          if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)__popc(mm));
-          wb = __shfl_sync(0xffffffffu, wb, 0);
-          if (h) {
-            const uint64_t pos = wb + __popc(mm & lt);
-            if (pos < (uint64_t)o.capacity) {
-              o.probe_idx[pos] = (int32_t)row[g + q];
-              o.build_idx[pos] = wi;
-              o.payload[pos] = wp;
-            }
+          if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)__popc(m));
+          wb = __shfl_sync(0xffffffffu, wb, 0) + __popc(m & lt);
+          const JoinVal v = p.side[i];
+          if ((side >> j & 1) && wb < cap) {
+            o.probe_idx[wb] = (int32_t)row(base, j);
+            o.build_idx[wb] = v.bidx;
+            o.payload[wb] = v.payload;
           }
         }
       }
     }
   }
+  if (EMIT && fill) flush();
   if (!EMIT) {
 #pragma unroll
     for (int off = 16; off; off >>= 1) counted += __shfl_xor_sync(0xffffffffu, counted, off);
@@ -268,22 +282,20 @@ rel_status join_launch_probe(const JoinParams& p, const JoinOut& o, const int64_
   const int id = emit ? relhost::K_JOIN_PROBE : relhost::K_JOIN_COUNT;
   // one wave of resident CTAs, each walking the tiles: a second, partial
   // wave would leave most SMs idle at the end
-  static int occ[2] = {0, 0};
-  int& o_ = occ[emit ? 1 : 0];
-  if (o_ == 0) {
-    const cudaError_t e0 =
-        emit ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o_, join_probe_fast_k<true>, J_BLOCK, 0)
-             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o_, join_probe_fast_k<false>, J_BLOCK, 0);
-    if (e0 != cudaSuccess || o_ < 1) o_ = 4;
-  }
-  const int64_t tiles = (n + (int64_t)J_BLOCK * J_IT - 1) / ((int64_t)J_BLOCK * J_IT);
-  int64_t g = (int64_t)relhost::device_sms() * o_;
+  // rows per thread: 1 while the rows do not fill the chip, whose warps then
+  // hold one lookup each (1e6 rows: 19 us against 24); above, 2 (4: spills or
+  // two CTAs per SM, 220 - 290 us against 202 for 16e6 rows)
+  const int u = n <= (int64_t)relhost::device_sms() * J_CTAS * J_BLOCK * 4 ? 1 : 2;
+  auto kern = emit ? (u == 1 ? join_probe_k<true, 1> : join_probe_k<true, 2>)
+                   : (u == 1 ? join_probe_k<false, 1> : join_probe_k<false, 2>);
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, J_BLOCK, 0) != cudaSuccess || occ < 1)
+    occ = J_CTAS;
+  const int64_t tile = (int64_t)J_BLOCK * u, tiles = (n + tile - 1) / tile;
+  int64_t g = (int64_t)relhost::device_sms() * occ;
   if (g > tiles) g = tiles;
   relhost::launch_begin(id, st);
-  if (emit)
-    join_probe_fast_k<true><<<(int)g, J_BLOCK, 0, st>>>(p, o, probe, n);
-  else
-    join_probe_fast_k<false><<<(int)g, J_BLOCK, 0, st>>>(p, o, probe, n);
+  kern<<<(int)g, J_BLOCK, 0, st>>>(p, o, probe, n);
   relhost::launch_end(id, st);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? REL_OK : relhost::cuda_fail(e, "launch(join probe)");

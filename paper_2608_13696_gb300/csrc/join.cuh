@@ -14,8 +14,8 @@ struct alignas(16) JoinVal {
 };
 
 // One slot of the single-call join table: the stored key (key ^ KEY_FLIP,
-// 0 = empty) and the build row index -- 16 bytes, read with one 128-bit
-// load.  The payload is gathered by that index from the table's own copy of
+// 0 = empty) and the build row index -- 16 bytes, read two at a time with one
+// 256-bit load.  The payload is gathered by that index from the table's own copy of
 // the payload column, so the L2-resident part of a 10^6-row table is 32 MB of
 // slots + 8 MB of payloads.
 struct alignas(16) JoinSlot {
