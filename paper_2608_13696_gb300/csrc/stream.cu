@@ -601,7 +601,12 @@ __global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constan
 // same for the partitions inside each bin.  Record order inside a partition
 // is arbitrary, which the aggregation does not see.
 // Two 256-thread CTAs per SM: while one waits at a barrier of its sort, the
-// other streams.
+// other streams.  The pinned keys' words are laid out as in gb_pin_k (three
+// loads and two stores a row, min and max stored only when they change) and
+// for the keys there are: 2e8 Zipf(1.1) rows, 8 pinned keys taking a third of
+// them, pass 2 with four words 1843 -> 1520 us (four 64-bit words each before,
+// 64 KB per CTA whatever the keys), with two words 1417; 2e8 uniform rows,
+// none pinned, 1364.  Reads and writes alone are 0.8 ms.
 constexpr int SP_BLOCK = 256;
 constexpr int SP_MIN_BLOCKS = 2;
 constexpr int SP_TILE = SP_BLOCK * ST_U;  // rows of one chunk, records sorted at once
@@ -611,6 +616,7 @@ static_assert(SP_BLOCK >= SP_BINS, "one thread per level-1 bin");
 // shared memory of pass 2 after the pinned words: bin counts, local and
 // global bases, bin ends, warp sums, then the tile's records and their bins
 constexpr size_t SP_SORT_SMEM = 4 * 4 * SP_BINS + 64 + 16 * SP_TILE + SP_TILE;
+constexpr uint32_t SP_HEAD = 416 + 8 * ST_PIN_LIMIT * 4;
 
 template <class KT, int NA, bool PIN, bool SCATTER>
 __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(const __grid_constant__ GbParams p) {
@@ -620,8 +626,14 @@ __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(con
   uint8_t* dense = sm + 256;
   uint64_t* pkd = (uint64_t*)(sm + 288);
   unsigned long long* csum = (unsigned long long*)(sm + 416);
-  uint64_t* acc = (uint64_t*)(sm + 416 + 8 * ST_PIN_LIMIT * 4);
-  uint8_t* const rest = (uint8_t*)(acc + ((PIN && SCATTER) ? PM * NA * SP_BLOCK : 0));
+  // thread-private words of the pinned keys there are, each [key][thread]:
+  // min and max side by side, sums, 32-bit counts
+  uint32_t n_hot = 0;
+  if (PIN && SCATTER)
+    for (uint32_t i = 0; i < p.tiny_slots; ++i) n_hot += p.tiny_init[i] != 0;
+  const uint32_t mm = smem_u32(sm) + SP_HEAD, sum = mm + (NA == 4 ? 16 : 0) * SP_BLOCK * n_hot,
+                 cnt = sum + 8 * SP_BLOCK * n_hot;
+  uint8_t* const rest = sm + SP_HEAD + (size_t)pk_key_bytes<NA>() * SP_BLOCK * n_hot;
   unsigned int* ctr = (unsigned int*)rest;  // pass 1: [P] counts
   // pass 2
   unsigned int* cnt1 = (unsigned int*)rest;
@@ -647,7 +659,7 @@ __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(con
       if (k != 0 && d < PM) pkd[d] = k;
     }
     if (SCATTER) {
-      for (int i = tid; i < PM * NA * SP_BLOCK; i += SP_BLOCK) acc[i] = 0;
+      for (uint32_t i = 4 * tid; i < pk_key_bytes<NA>() * SP_BLOCK * n_hot; i += 4 * SP_BLOCK) sts32(mm + i, 0);
       for (int i = tid; i < PM * NA; i += SP_BLOCK) csum[i] = 0;
     }
   }
@@ -729,14 +741,18 @@ __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(con
 #pragma unroll
         for (int j = 0; j < ST_U; ++j) {
           if (!(pinm >> j & 1)) continue;
-          uint64_t w[NA];
-          words_of<NA>(val[j], w);
-          uint64_t* t = acc + (size_t)dd[j] * NA * SP_BLOCK + tid;
-#pragma unroll
-          for (int a = 0; a < NA; ++a) {
-            const uint64_t o = t[a * SP_BLOCK];
-            t[a * SP_BLOCK] = umax_word<NA>(a) ? (o > w[a] ? o : w[a]) : o + w[a];
+          const uint32_t at = dd[j] * SP_BLOCK + tid;
+          const uint64_t o = lds64(sum + 8 * at);
+          const uint32_t c = lds32(cnt + 4 * at);
+          if constexpr (NA == 4) {
+            uint64_t mn, mx;
+            lds128(mm + 16 * at, mn, mx);
+            const uint64_t lo = val[j] ^ MIN_FLIP, hi = val[j] ^ MAX_FLIP;
+            if (lo > mn) sts64(mm + 16 * at, lo);
+            if (hi > mx) sts64(mm + 16 * at + 8, hi);
           }
+          sts64(sum + 8 * at, o + val[j]);
+          sts32(cnt + 4 * at, c + 1);
         }
       }
     }
@@ -837,10 +853,12 @@ __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(con
     return;
   }
   if (PIN) {
-    for (int d = 0; d < PM; ++d) {
+    for (uint32_t d = 0; d < n_hot; ++d) {
 #pragma unroll
       for (int a = 0; a < NA; ++a) {
-        uint64_t x = acc[((size_t)d * NA + a) * SP_BLOCK + tid];
+        const uint32_t at = d * SP_BLOCK + tid;
+        uint64_t x = a == 0 ? lds64(sum + 8 * at) : a == 1 ? (uint64_t)lds32(cnt + 4 * at)
+                                                           : lds64(mm + 16 * at + 8 * (a - 2));
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
           const uint64_t y = __shfl_xor_sync(0xffffffffu, x, o);
@@ -864,17 +882,19 @@ __global__ void __launch_bounds__(SP_BLOCK, SP_MIN_BLOCKS) gb_ppass_stream_k(con
   }
 }
 
-size_t ppass_smem(int na, bool pin, bool scatter, uint32_t part_bits) {
-  size_t b = 416 + 8 * ST_PIN_LIMIT * 4;
-  if (pin && scatter) b += (size_t)8 * (na == 4 ? pin_max<4>() : pin_max<2>()) * na * SP_BLOCK;
-  return b + (scatter ? SP_SORT_SMEM : 4ull * (1u << part_bits));
+size_t ppass_smem(const GbParams& p, int na, bool pin, bool scatter) {
+  size_t b = SP_HEAD;
+  if (pin && scatter)
+    for (uint32_t i = 0; i < p.tiny_slots; ++i)
+      if (p.tiny_init[i] != 0) b += (size_t)(na == 4 ? pk_key_bytes<4>() : pk_key_bytes<2>()) * SP_BLOCK;
+  return b + (scatter ? SP_SORT_SMEM : 4ull << p.part_bits);
 }
 
 // CTAs of a pass that fit on the SMs at once (at most cap), or 0.
 template <class KT, int NA, bool PIN, bool SCATTER>
 uint32_t ppass_grid(const GbParams& p, uint32_t cap) {
   auto kern = gb_ppass_stream_k<KT, NA, PIN, SCATTER>;
-  const size_t smem = ppass_smem(NA, PIN, SCATTER, p.part_bits);
+  const size_t smem = ppass_smem(p, NA, PIN, SCATTER);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 0;
   int occ = 0;
@@ -890,7 +910,7 @@ uint32_t ppass_grid(const GbParams& p, uint32_t cap) {
 template <class KT, int NA, bool PIN, bool SCATTER>
 rel_status launch_ppass(const GbParams& p, cudaStream_t st) {
   auto kern = gb_ppass_stream_k<KT, NA, PIN, SCATTER>;
-  const size_t smem = ppass_smem(NA, PIN, SCATTER, p.part_bits);
+  const size_t smem = ppass_smem(p, NA, PIN, SCATTER);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(partition pass)");
   const uint32_t grid = SCATTER ? ppass_grid<KT, NA, PIN, SCATTER>(p, 1u << 16) : p.fixed_grid;
@@ -1130,8 +1150,8 @@ bool gb_ppass_stream_eligible(const GbParams& p, int shape, int n_hot) {
   const int na = (shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32) ? 4 : 2;
   const int pmax = na == 4 ? pin_max<4>() : pin_max<2>();
   if (p.tiny_slots && !(p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= pmax)) return false;
-  return ppass_smem(na, p.tiny_slots != 0, true, p.part_bits) * SP_MIN_BLOCKS <= 227 * 1024 &&
-         ppass_smem(na, p.tiny_slots != 0, false, p.part_bits) * SP_MIN_BLOCKS <= 227 * 1024;
+  return ppass_smem(p, na, p.tiny_slots != 0, true) * SP_MIN_BLOCKS <= 227 * 1024 &&
+         ppass_smem(p, na, p.tiny_slots != 0, false) * SP_MIN_BLOCKS <= 227 * 1024;
 }
 
 rel_status gb_launch_ppass_stream(const GbParams& p, int shape, bool scatter, cudaStream_t st) {
