@@ -19,8 +19,9 @@
 // per-CTA tables merge into the global one at the end, so every layer
 // configuration yields the same exact groups.  A compaction kernel turns
 // occupied slots into dense output rows (warp ballot / popc, one atomic per
-// warp).  Runs the fused filter + aggregate shape (ShapeQ1) and plans with a
-// staging ring of their own; gen.cu and stream.cu have the other shapes.
+// warp).  Runs the fused filter + aggregate shape (ShapeQ1) where its keys are
+// not all pinned (q1.cu has those) and plans with a staging ring of their own;
+// gen.cu and stream.cu have the other shapes.
 #include "groupby.cuh"
 #include "smtab.cuh"
 

@@ -35,7 +35,7 @@ constexpr int PART_MAX_BITS = 14;  // at most 16384 partitions
 // records by destination in shared memory and write each destination's run
 // contiguously.
 constexpr int PART_L1_BITS = 8;
-constexpr int PART_TILE = 4096;
+constexpr int PART_TILE = 2048;
 
 // Row shapes.  The specialised ones fix column types and aggregate kinds at
 // compile time; KV4 / KV2 hold their aggregates in the internal order

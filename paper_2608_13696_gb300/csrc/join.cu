@@ -231,19 +231,19 @@ __global__ void __launch_bounds__(J_BLOCK, J_CTAS) join_probe_k(const __grid_con
       for (int j = 0; j < U; ++j) {
         const unsigned m = __ballot_sync(0xffffffffu, side >> j & 1);
         if (!m) continue;
-        if (!EMIT) {
+        if constexpr (!EMIT) {
           counted += side >> j & 1 ? n_side : 0;
-          continue;
-        }
-        for (uint64_t i = 0; i < n_side; ++i) {
-          unsigned long long wb = 0;
-          if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)__popc(m));
-          wb = __shfl_sync(0xffffffffu, wb, 0) + __popc(m & lt);
-          const JoinVal v = p.side[i];
-          if ((side >> j & 1) && wb < cap) {
-            o.probe_idx[wb] = (int32_t)row(base, j);
-            o.build_idx[wb] = v.bidx;
-            o.payload[wb] = v.payload;
+        } else {
+          for (uint64_t i = 0; i < n_side; ++i) {
+            unsigned long long wb = 0;
+            if (lane == 0) wb = atomicAdd(&p.hdr->n_out, (unsigned long long)__popc(m));
+            wb = __shfl_sync(0xffffffffu, wb, 0) + __popc(m & lt);
+            const JoinVal v = p.side[i];
+            if ((side >> j & 1) && wb < cap) {
+              o.probe_idx[wb] = (int32_t)row(base, j);
+              o.build_idx[wb] = v.bidx;
+              o.payload[wb] = v.payload;
+            }
           }
         }
       }

@@ -3,20 +3,21 @@
 // KV2 of the fused kernel, without its staging ring.
 //
 // The paper's group-by kernels are issue-bound (Sec. 5, 7): instructions per
-// DRAM sector, not bandwidth, limit them.  This kernel keeps the per-row path
-// short.  Rows come straight from HBM in 16-byte vector loads (two rows per
-// load and column, ST_U rows per thread per chunk, evict-first), so a thread
-// has 2 x ST_U / 2 loads in flight and no shared-memory staging or barrier
-// sits on the path.  Each row then goes to the first layer that takes it:
-//  * pinned hot keys (from the sample sketch): a one-probe perfect-hash test
-//    against the pinned key, then thread-private accumulators in shared
-//    memory (one column per thread: no atomics, no bank conflicts);
-//  * the global table: every row still unplaced issues its first slot read
-//    before any is resolved (ST_U independent L2 round trips per thread),
-//    then claims or accumulates with CAS / RED atomics, bounded probing.
-// At the end each CTA folds its thread-private words (warp shuffles, then
-// shared atomics) into the global table, which the compaction kernel turns
-// into the output.  Plans with CTA-shared slots run gb_smem_k instead.
+// DRAM sector, not bandwidth, limit them.  The kernels here keep the per-row
+// path short.  Rows come straight from HBM in 16-byte vector loads (two rows per
+// load and column, several rows per thread in flight, evict-first), with no
+// shared-memory staging or barrier on the path.  By what the plan has:
+//  * gb_smem_k: a CTA-shared table (smtab.cuh), the global one behind it;
+//  * gb_pin_k: pinned hot keys (from the sample sketch) that are all the keys
+//    there are: a one-probe perfect-hash test, then thread-private words in
+//    shared memory (one column per thread: no atomics, no bank conflicts);
+//  * gb_stream_k: pinned keys and others, whose rows issue their first slot read
+//    of the global table before any is resolved, then claim or accumulate with
+//    CAS / RED atomics, bounded probing;
+//  * gb_glob_k: the global table alone;
+//  * gb_ppass_stream_k and gb_part_l2_k: the partitioned plans' passes.
+// At the end a CTA folds its own words into the global table, which the
+// compaction kernel turns into the output.
 #include "groupby.cuh"
 #include "smtab.cuh"
 
@@ -1008,13 +1009,17 @@ bool gb_stream_shape(int shape) {
 // (tiles never straddle a bin) is sorted by partition inside its bin in
 // shared memory; each partition's run is claimed with one atomic on the
 // partition's cursor and written contiguously.  Persistent grid; tile t
-// belongs to the last bin b with l2_tiles[b] <= t.
-constexpr int L2_BLOCK = 512;
+// belongs to the last bin b with l2_tiles[b] <= t.  Bound by its shared memory
+// (ranks by atomics, the records' scattered stores) and by the barriers between:
+// four CTAs of 256 threads and 2048 records per SM rather than two of 512 and
+// 4096, 942 -> 872 us for the 1.4e8 records of 2e8 Zipf(1.1) rows and 1246 ->
+// 1144 for 2e8 uniform ones (reads and writes alone: 0.66 and 0.94 ms).
+constexpr int L2_BLOCK = 256;
 constexpr int L2_U = PART_TILE / L2_BLOCK;
 constexpr int L2_MAX_SUB = 1 << (PART_MAX_BITS - PART_L1_BITS);
 constexpr size_t L2_SMEM = 16 * PART_TILE + PART_TILE;
 
-__global__ void __launch_bounds__(L2_BLOCK, 2) gb_part_l2_k(const __grid_constant__ GbParams p) {
+__global__ void __launch_bounds__(L2_BLOCK, 4) gb_part_l2_k(const __grid_constant__ GbParams p) {
   extern __shared__ __align__(16) uint8_t sm[];
   PartRec* recbuf = (PartRec*)sm;
   uint8_t* slot_bin = sm + 16 * PART_TILE;
