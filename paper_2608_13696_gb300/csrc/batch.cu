@@ -486,31 +486,40 @@ __device__ __forceinline__ int64_t decode_word(int op, uint64_t w) {
   return op == REL_MIN ? (int64_t)(w ^ MIN_FLIP) : op == REL_MAX ? (int64_t)(w ^ MAX_FLIP) : (int64_t)w;
 }
 
+// Compaction of a tile of slots: a thread's ITEMS keys are read together and a
+// warp takes one output claim for all of them.
 template <int ITEMS>
 __device__ __forceinline__ void compact_tile(const BatchGb& g, BatchStatus* st, long long t) {
   const int B = blockDim.x;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const long long slots = 1ll << g.log2_slots;
-  const long long s0 = t * (long long)B * ITEMS;
+  const long long s0 = t * (long long)B * ITEMS + threadIdx.x;
+  uint64_t k[ITEMS];
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
-    const long long s = s0 + (long long)j * B + threadIdx.x;
-    const uint64_t k = s < slots ? g.tkeys[s] : 0;
-    const unsigned m = __ballot_sync(0xffffffffu, k != 0);
-    if (!m) continue;
+    const long long s = s0 + (long long)j * B;
+    k[j] = s < slots ? g.tkeys[s] : 0;
+  }
+  uint32_t total = 0;
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) total += __popc(__ballot_sync(0xffffffffu, k[j] != 0));
+  if (total) {
     unsigned long long wb = 0;
-    if (lane == 0) wb = atomicAdd(&st->n_out, (unsigned long long)__popc(m));
+    if (lane == 0) wb = atomicAdd(&st->n_out, (unsigned long long)total);
     wb = __shfl_sync(0xffffffffu, wb, 0);
-    if (k != 0) {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const unsigned m = __ballot_sync(0xffffffffu, k[j] != 0);
       const unsigned long long pos = wb + __popc(m & lt);
-      if (pos < (unsigned long long)g.out_capacity) {
-        g.out_keys[pos] = (int64_t)(k ^ KEY_FLIP);
-        const unsigned long long* w = g.taggs + (uint64_t)s * g.n_aggs;
+      if (k[j] != 0 && pos < (unsigned long long)g.out_capacity) {
+        g.out_keys[pos] = (int64_t)(k[j] ^ KEY_FLIP);
+        const unsigned long long* w = g.taggs + (uint64_t)(s0 + (long long)j * B) * g.n_aggs;
 #pragma unroll
         for (int a = 0; a < BATCH_MAX_AGGS; ++a)
           if (a < g.n_aggs) g.out_aggs[a][pos] = decode_word(g.ops[a], w[a]);
       }
+      wb += __popc(m);
     }
   }
   if (t == 0 && threadIdx.x == 0 && st->n_side > 0) {
@@ -648,9 +657,11 @@ __device__ __forceinline__ void probe_tile(const BatchJoin& J, BatchStatus* st, 
   probe_rows(J, st, r0, r0 + rows < J.n_probe ? r0 + rows : J.n_probe);
 }
 
-// Persistent launch B: join probes, then group-by compaction.
+// Persistent launch B: join probes, then group-by compaction.  Three CTAs per
+// SM: both halves wait on L2 round trips (512 group-bys and 64 joins, 512 x 4:
+// 812 -> 712 us against two CTAs, in spite of 56 bytes of spills).
 template <int ITEMS>
-__global__ void __launch_bounds__(512) batch_b(const __grid_constant__ BatchArgs a) {
+__global__ void __launch_bounds__(512, 3) batch_b(const __grid_constant__ BatchArgs a) {
   __shared__ long long s_item;
   __shared__ int s_inst;
   __shared__ union {

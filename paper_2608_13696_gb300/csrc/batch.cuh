@@ -14,7 +14,7 @@ constexpr int BATCH_MAX_SMEM_SLOTS = 4096;
 // descriptor copy, clearing and flushing a shared-memory table) are paid once
 // per ~64K rows rather than once per tile.
 constexpr int BATCH_GB_SPAN = 32;
-// ... and of one probe work item.
+// ... and of one probe work item, at most.
 constexpr int BATCH_JOIN_SPAN = 8;
 
 // One group-by instance as the kernels see it.
