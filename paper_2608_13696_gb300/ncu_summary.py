@@ -36,11 +36,11 @@ SOURCES = {
     "gb_part_scatter": ["stream.cu", "api.cu"],
     "gb_part_l2": ["stream.cu", "api.cu"],
     "gb_part_scan": ["groupby.cu", "api.cu"],
-    "gb_part_agg": ["groupby.cu", "api.cu"],
+    "gb_part_agg": ["groupby.cu", "smtab.cuh", "api.cu"],
     "gb_compact": ["groupby.cu", "api.cu"],
     "gb_main_regs": ["groupby.cu", "api.cu"],
-    "gb_main_layered": ["groupby.cu", "api.cu"],
-    "gb_main_staged_keyset": ["groupby.cu", "api.cu"],
+    "gb_main_layered": ["q1.cu", "api.cu"],
+    "gb_main_staged_keyset": ["gen.cu", "api.cu"],
     "gb_stream": ["stream.cu", "api.cu"],
     "join_build": ["join.cu", "api.cu"],
     "join_probe": ["join.cu", "api.cu"],
@@ -49,7 +49,7 @@ SOURCES = {
     "mlp_backward_sample": ["mlp.cu", "api.cu"],
     "mlp_backward": ["mlp.cu", "api.cu"],
     "mlp_adamw": ["mlp.cu", "api.cu"],
-    "batch_a": ["batch.cu", "batch_api.cu"],
+    "batch_a": ["batch.cu", "smtab.cuh", "batch_api.cu"],
     "batch_b": ["batch.cu", "batch_api.cu"],
     "shard_scatter": ["shard.cu"],
     "hll": ["distinct.cu", "api.cu"],

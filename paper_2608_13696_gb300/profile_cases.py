@@ -8,11 +8,11 @@ CASE (inputs seeded and synthetic, as in the bench):
   part      partitioned group-by of 5e7 Zipf(1.1) key/value rows with the
             sample sketch's pins (histogram, scan, two scatter levels,
             aggregation, compaction)
-  stream    streaming group-by of 5e7 four-key rows with pinned keys (gb_stream)
+  stream    streaming group-by of 5e7 four-key rows, all keys pinned (gb_pin_k)
   join      join build of 1e6 unique keys and probe of 1.6e7 keys (90 % hits)
-  lineitem  fused filter + group-by of 2e7 lineitem rows: exact count (staged
-            key set), sketch, aggregation in thread-private shared words,
-            compaction
+  lineitem  fused filter + group-by of 2e7 lineitem rows: exact count (one
+            bit per packed key, gb_gen_bits_k), sketch, aggregation in
+            thread-private shared words (gb_q1_k), compaction
   mlp       planner network forward, backward and AdamW on a batch of 256
   batch     a batch of 512 group-bys and 64 join partitions (the batched
             workload's recipe, rows divided by 8): the two persistent launches
