@@ -709,8 +709,7 @@ rel_status launch_pair(const BatchArgs& a, int block, int smem, int grid_a, int 
 
 template <int ITEMS, int W>
 rel_status occ_pair(int block, int smem, int* pa, int* pb) {
-  cudaError_t e = cudaFuncSetAttribute(batch_a<ITEMS, W>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = relhost::allow_smem(batch_a<ITEMS, W>);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(batch)");
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pa, batch_a<ITEMS, W>, block, smem);
   if (e == cudaSuccess)

@@ -445,7 +445,7 @@ template <class K>
 rel_status launch_gen(K kern, int id, size_t smem, const GbParams& p, cudaStream_t st,
                       bool beside = false) {
   if (p.n_rows == 0) return REL_OK;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = relhost::allow_smem(kern);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(generic)");
   // 1024 resident threads per SM (64 registers each) whatever the table's
   // size; small inputs in small CTAs, so that more SMs take part

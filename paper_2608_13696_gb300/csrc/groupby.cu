@@ -1216,10 +1216,8 @@ template <class S, class BE, bool TMA>
 int occupancy(const GbParams& p) {
   auto kern = gb_main<S, BE, TMA>;
   const size_t smem = smem_of<S, BE, TMA>(p);
-  if (smem > 227 * 1024) return 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return 0;
+  if (smem > (size_t)relhost::CTA_SMEM) return 0;
+  if (relhost::allow_smem(kern, 0) != cudaSuccess) return 0;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GB_THREADS, smem) != cudaSuccess)
     return 0;
@@ -1325,8 +1323,7 @@ rel_status gb_launch_part_scan(const GbParams& p, bool cta_offsets, cudaStream_t
     gb_part_sum<<<(P + 7) / 8, 256, 0, st>>>(p);
   relhost::launch_end(relhost::K_GB_PSCAN, st);
   const int smem = (int)(4 * (P + P / 32));
-  const cudaError_t e0 =
-      cudaFuncSetAttribute(gb_part_scan2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e0 = relhost::allow_smem(gb_part_scan2);
   if (e0 != cudaSuccess) return relhost::cuda_fail(e0, "cudaFuncSetAttribute(partition scan)");
   relhost::launch_begin(relhost::K_GB_PSCAN, st);
   gb_part_scan2<<<1, 1024, smem, st>>>(p);
@@ -1341,7 +1338,7 @@ template <int NA>
 rel_status launch_part_agg(const GbParams& p, const GbOut& o, cudaStream_t st) {
   auto kern = gb_part_agg<NA>;
   const size_t smem = SmTab<NA>::bytes(p.smem_slots);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = relhost::allow_smem(kern);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(partition agg)");
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GB_BLOCK, smem);

@@ -188,7 +188,7 @@ rel_status gb_launch_q1(const GbParams& p, int n_hot, cudaStream_t st) {
   int block = p.n_rows > (int64_t)relhost::device_sms() * 4096 ? 768 : 256;
   while (block > 128 && q1_smem(n_hot, block) > 184 * 1024) block -= 128;
   const size_t smem = q1_smem(n_hot, block);
-  cudaError_t e = cudaFuncSetAttribute(gb_q1_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = relhost::allow_smem(gb_q1_k);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(fused)");
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gb_q1_k, block, smem);

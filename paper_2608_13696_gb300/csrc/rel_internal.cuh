@@ -282,6 +282,16 @@ enum KernelId : int {
 void launch_begin(int kernel_id, cudaStream_t st);
 void launch_end(int kernel_id, cudaStream_t st);
 
+// Let a kernel use all the shared memory of a CTA that its own variables leave
+// (at most own_bytes of them).  The limit belongs to the kernel, not to a
+// launch: one that follows each plan's size is lowered by another thread's
+// smaller plan, or by another batch's, before a launch that needs more of it.
+constexpr int CTA_SMEM = 227 * 1024;
+template <class K>
+cudaError_t allow_smem(K kern, int own_bytes = 12 * 1024) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CTA_SMEM - own_bytes);
+}
+
 // Launch a kernel; beside: it may start before the kernel in front of it in
 // the stream has finished (it must not read what that one writes, and ends
 // with wait_for_earlier_kernels).

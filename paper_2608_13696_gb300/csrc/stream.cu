@@ -896,7 +896,7 @@ template <class KT, int NA, bool PIN, bool SCATTER>
 uint32_t ppass_grid(const GbParams& p, uint32_t cap) {
   auto kern = gb_ppass_stream_k<KT, NA, PIN, SCATTER>;
   const size_t smem = ppass_smem(p, NA, PIN, SCATTER);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (relhost::allow_smem(kern) != cudaSuccess)
     return 0;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, SP_BLOCK, smem) != cudaSuccess)
@@ -912,7 +912,7 @@ template <class KT, int NA, bool PIN, bool SCATTER>
 rel_status launch_ppass(const GbParams& p, cudaStream_t st) {
   auto kern = gb_ppass_stream_k<KT, NA, PIN, SCATTER>;
   const size_t smem = ppass_smem(p, NA, PIN, SCATTER);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = relhost::allow_smem(kern);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(partition pass)");
   const uint32_t grid = SCATTER ? ppass_grid<KT, NA, PIN, SCATTER>(p, 1u << 16) : p.fixed_grid;
   if (grid < 1) return relhost::set_error("group-by: partition pass does not fit"), REL_E_UNSUPPORTED;
@@ -940,7 +940,7 @@ size_t stream_smem(int na) {
 template <class K>
 rel_status launch_rows(K kern, int block, size_t smem, int64_t chunk, const GbParams& p,
                        cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = relhost::allow_smem(kern);
   if (e != cudaSuccess) return relhost::cuda_fail(e, "cudaFuncSetAttribute(stream)");
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem);
