@@ -417,10 +417,16 @@ constexpr uint32_t PART_MAX_GRID = PART_HIST_COLS - 1;  // CTAs of the histogram
 // records into equal pieces instead of taking whole partitions: 256
 // partitions would occupy 256 of its ~600 CTAs.
 constexpr int PART_SPLIT_BITS = 8;
-// the most groups that 256 partitions (one scatter level) take, 1172 to a
-// 2048-slot table (four aggregates, 250000
-// groups: 2.5e7 rows 0.69 -> 0.56 ms, 1e8 2.43 -> 1.86)
-constexpr int64_t PART_ONE_LEVEL_GROUPS = 300000;
+// the most groups that 256 partitions (one scatter level) take, 1024 to a
+// 2048-slot table, the same table slots in all as 512 partitions of 1024 (four
+// aggregates, 250000 groups: 2.5e7 rows 0.69 -> 0.56 ms, 1e8 2.43 -> 1.86)
+constexpr int64_t PART_ONE_LEVEL_GROUPS = 262144;
+
+// Key/value plans of more than 2048 groups: the fewest slots of the global
+// table, whatever the variant.  A hint, or an estimate from a sample, may be
+// low by some times; the table then still holds the groups (65536 slots: 2.6 MB
+// to clear and scan with four aggregates).
+constexpr int64_t MIN_SPILL_SLOTS = 65536;
 
 bool part_shape(int shape) {
   return shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 || shape == SHAPE_KV2_64 ||
@@ -544,7 +550,7 @@ void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
   if (2 * keys_per_part > (uint64_t)plan->smem_slots) spill = 2 * (uint64_t)est;
   // few partitions: their pieces meet in the global table (part_split)
   if (bits <= PART_SPLIT_BITS) spill = std::max(spill, (uint64_t)plan->smem_slots << bits);
-  plan->slots = (int64_t)next_pow2(spill > 65536 ? spill : 65536);
+  plan->slots = (int64_t)next_pow2(std::max(spill, (uint64_t)MIN_SPILL_SLOTS));
   (void)n_rows;
 }
 
@@ -886,7 +892,11 @@ void choose_variant(int variant, int64_t est, int64_t n_rows, int words, bool p_
       break;
     default:
       choose_layers(est, words, plan);
-      if (plan->variant == REL_VAR_GLOBAL && p_ok) choose_partitioned(est, n_rows, plan);
+      if (!p_ok) break;
+      if (plan->variant == REL_VAR_GLOBAL)
+        choose_partitioned(est, n_rows, plan);
+      else if (est > 2048)
+        plan->slots = std::max(plan->slots, MIN_SPILL_SLOTS);
   }
 }
 
@@ -1123,7 +1133,7 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
     if (!forced && prefer_global(info, d->n_rows, plan)) {
       plan->variant = REL_VAR_GLOBAL;
       plan->part_bits = plan->smem_slots = plan->tiny_slots = 0;
-      plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
+      plan->slots = std::max((int64_t)next_pow2((uint64_t)(2 * est)), MIN_SPILL_SLOTS);
     }
   }
   plan->workspace_bytes = plan_ws_bytes(plan, d->n_aggs, d->n_rows);
@@ -1307,7 +1317,7 @@ uint64_t rel_groupby_auto_ws_bytes(const rel_groupby_desc* d) {
   // every estimate is at most n_rows
   const uint64_t n = (uint64_t)d->n_rows;
   const uint64_t slots = next_pow2(2 * n < 16 ? 16 : 2 * n);
-  const uint64_t p_slots = next_pow2(2 * n > 65536 ? 2 * n : 65536);
+  const uint64_t p_slots = next_pow2(std::max(2 * n, (uint64_t)MIN_SPILL_SLOTS));
   uint64_t need = gb_ws_bytes((int64_t)slots, d->n_aggs);
   need = std::max(need, part_layout((int64_t)p_slots, d->n_aggs, PART_MAX_BITS, d->n_rows).end);
   need = std::max(need, HEADER_BYTES + 8 * slots);  // exact pre-pass key set
