@@ -413,10 +413,20 @@ constexpr uint32_t PART_HIST_COLS = 512;                 // columns of the histo
 constexpr uint32_t PART_MAX_GRID = PART_HIST_COLS - 1;  // CTAs of the histogram / scatter passes
                                                         // (the last column holds part_extra)
 
-// With at most 2^PART_SPLIT_BITS partitions the aggregation pass cuts the
+// With at most 2^PART_SPLIT_BITS partitions the aggregation pass may cut the
 // records into equal pieces instead of taking whole partitions: 256
-// partitions would occupy 256 of its ~600 CTAs.
+// partitions would occupy 256 of its ~600 CTAs.  The pieces meet in the global
+// table, key by key, so that it pays only where a partition has the rows for it:
+// keys without skew (a sketch pinned none) want the more the more partitions
+// there are (four aggregates, rows at which both take the same time: 16
+// partitions 1e5, 64 1e6, 256 1.2e7; half of that 5-20 % more time in pieces);
+// skewed ones, whose whole partitions are uneven, 8000 a partition or a little
+// more (without pins 2000), and what is not known is taken for skewed.
 constexpr int PART_SPLIT_BITS = 8;
+
+bool split_pays(int bits, int64_t n_rows, bool flat) {
+  return bits <= PART_SPLIT_BITS && n_rows >> bits >= (flat ? 4000 + (200ll << bits) : 8000);
+}
 // the most groups that 256 partitions (one scatter level) take, 1024 to a
 // 2048-slot table, the same table slots in all as 512 partitions of 1024 (four
 // aggregates, 250000 groups: 2.5e7 rows 0.69 -> 0.56 ms, 1e8 2.43 -> 1.86)
@@ -480,7 +490,7 @@ rel_status run_partitioned(GbParams& p, const rel_plan* plan, int shape, const G
   p.part_extra = (unsigned int*)p.hist + ((size_t)PART_MAX_GRID << p.part_bits);
   p.recs = (PartRec*)(base + L.recs);
   p.recs1 = p.part_bits > PART_L1_BITS ? (PartRec*)(base + L.recs1) : nullptr;
-  p.part_split = plan->part_bits <= PART_SPLIT_BITS &&
+  p.part_split = split_pays(plan->part_bits, p.n_rows, (plan->flags & REL_PLAN_SKETCH) && plan->n_hot == 0) &&
                  plan->slots >= (int64_t)plan->smem_slots << plan->part_bits;
   uint32_t grid = 2u * (uint32_t)relhost::device_sms();
   p.fixed_grid = grid > PART_MAX_GRID ? PART_MAX_GRID : grid;
@@ -525,12 +535,15 @@ rel_status run_partitioned(GbParams& p, const rel_plan* plan, int shape, const G
 }
 
 // Many groups over key + value rows: partition instead of one big table.
-void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
+// flat: a sketch showed no skew.
+void choose_partitioned(int64_t est, int64_t n_rows, bool flat, rel_plan* plan) {
   uint64_t per = (uint64_t)(est / 768);
   int bits = 4;
   while (bits < PART_MAX_BITS && (1ull << bits) < per) ++bits;
   // a little past one scatter level: larger tables instead of the second level
-  const bool larger = bits == PART_L1_BITS + 1 && est <= PART_ONE_LEVEL_GROUPS;
+  // (which leave the aggregation fewer partitions than CTAs: only in pieces)
+  const bool larger = bits == PART_L1_BITS + 1 && est <= PART_ONE_LEVEL_GROUPS &&
+                      split_pays(PART_L1_BITS, n_rows, flat);
   if (larger) bits = PART_L1_BITS;
   plan->variant = REL_VAR_PARTITIONED;
   plan->part_bits = bits;
@@ -548,10 +561,9 @@ void choose_partitioned(int64_t est, int64_t n_rows, rel_plan* plan) {
   // (more keys per partition than half a table of the largest size)
   uint64_t spill = (uint64_t)est / 4;
   if (2 * keys_per_part > (uint64_t)plan->smem_slots) spill = 2 * (uint64_t)est;
-  // few partitions: their pieces meet in the global table (part_split)
-  if (bits <= PART_SPLIT_BITS) spill = std::max(spill, (uint64_t)plan->smem_slots << bits);
+  // their pieces meet in the global table
+  if (split_pays(bits, n_rows, flat)) spill = std::max(spill, (uint64_t)plan->smem_slots << bits);
   plan->slots = (int64_t)next_pow2(std::max(spill, (uint64_t)MIN_SPILL_SLOTS));
-  (void)n_rows;
 }
 
 // Per-CTA layers for an expected number of groups.
@@ -615,18 +627,23 @@ int32_t tiny_capacity(int words) {
   return words <= 2 ? 32 : words <= 4 ? 16 : words <= 6 ? 8 : 0;
 }
 
+// The sample's eight most frequent keys hold 5 % of its rows.
+bool skewed(const rel_sketch_info& s) {
+  int64_t top8 = 0;
+  for (int i = 0; i < 8; ++i) top8 += s.top_count[i];
+  return top8 * 20 >= (int64_t)s.kept;
+}
+
 // Pin the sample's frequent keys: all of them when the plan keeps every group
 // thread-private, else the heavy hitters of a skewed sample.
 void apply_sketch(const rel_sketch_info& s, int words, rel_plan* plan) {
   const int32_t cap = tiny_capacity(words);
   if (cap == 0 || s.kept == 0) return;
-  int64_t top8 = 0;
-  for (int i = 0; i < 8; ++i) top8 += s.top_count[i];
   const bool tiny_only = plan->tiny_slots && !plan->smem_slots;
   int want = 0;
   if (tiny_only) {
     want = s.ndv < plan->tiny_slots ? s.ndv : plan->tiny_slots;
-  } else if (top8 * 20 >= (int64_t)s.kept) {  // top 8 keys hold >= 5 % of rows
+  } else if (skewed(s)) {
     plan->tiny_slots = cap;
     for (int i = 0; i < REL_SKETCH_TOP && i < cap / 2; ++i)
       if (s.top_count[i] >= 2) want = i + 1;
@@ -871,7 +888,7 @@ uint64_t batched_plan_out_off(int32_t n) {
 }
 
 // Table layers for a variant (0 = the rule by group count).
-void choose_variant(int variant, int64_t est, int64_t n_rows, int words, bool p_ok,
+void choose_variant(int variant, int64_t est, int64_t n_rows, int words, bool p_ok, bool flat,
                     rel_plan* plan) {
   switch (variant) {
     case REL_VAR_SMEM:
@@ -888,13 +905,13 @@ void choose_variant(int variant, int64_t est, int64_t n_rows, int words, bool p_
       plan->smem_slots = 0;
       break;
     case REL_VAR_PARTITIONED:
-      choose_partitioned(est, n_rows, plan);
+      choose_partitioned(est, n_rows, flat, plan);
       break;
     default:
       choose_layers(est, words, plan);
       if (!p_ok) break;
       if (plan->variant == REL_VAR_GLOBAL)
-        choose_partitioned(est, n_rows, plan);
+        choose_partitioned(est, n_rows, flat, plan);
       else if (est > 2048)
         plan->slots = std::max(plan->slots, MIN_SPILL_SLOTS);
   }
@@ -1113,22 +1130,23 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
   } else {
     est = d->n_rows;
   }
+  const bool sketch = (flags & REL_PLAN_SKETCH) && d->n_rows > 0;
+  if (sketch && !have_info) {
+    const uint64_t need = rel_sketch_ws_bytes();
+    if (plan->scratch_bytes < need) plan->scratch_bytes = need;
+    if (!ws || ws_bytes < plan->scratch_bytes) {
+      set_error("plan: sketching needs %llu workspace bytes",
+                (unsigned long long)plan->scratch_bytes);
+      return REL_E_CAPACITY;
+    }
+    if ((r = rel_sketch(d, ws, ws_bytes, &info, st))) return r;
+  }
   plan->est_groups = est;
   plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
   // (a network that prefers the global table leaves the choice to the rules)
   choose_variant(forced ? forced : learned == REL_VAR_GLOBAL ? 0 : learned, est, d->n_rows,
-                 gb_shape_width(m.shape), p_ok, plan);
-  if ((flags & REL_PLAN_SKETCH) && d->n_rows > 0) {
-    if (!have_info) {
-      const uint64_t need = rel_sketch_ws_bytes();
-      if (plan->scratch_bytes < need) plan->scratch_bytes = need;
-      if (!ws || ws_bytes < plan->scratch_bytes) {
-        set_error("plan: sketching needs %llu workspace bytes",
-                  (unsigned long long)plan->scratch_bytes);
-        return REL_E_CAPACITY;
-      }
-      if ((r = rel_sketch(d, ws, ws_bytes, &info, st))) return r;
-    }
+                 gb_shape_width(m.shape), p_ok, sketch && !skewed(info), plan);
+  if (sketch) {
     apply_sketch(info, gb_shape_width(m.shape), plan);
     if (!forced && prefer_global(info, d->n_rows, plan)) {
       plan->variant = REL_VAR_GLOBAL;
@@ -1480,7 +1498,7 @@ rel_status rel_plan_size_batched(const rel_groupby_desc* descs, int32_t n, uint3
     learned_rule(info[i], &y[(size_t)i * REL_MLP_OUT], d->n_rows, false, &est, &variant);
     plan->est_groups = est;
     plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
-    choose_variant(variant, est, d->n_rows, gb_shape_width(m.shape), false, plan);
+    choose_variant(variant, est, d->n_rows, gb_shape_width(m.shape), false, false, plan);
     plan->workspace_bytes = plan_ws_bytes(plan, d->n_aggs, d->n_rows);
     if (flags & REL_PLAN_SKETCH) apply_sketch(info[i], gb_shape_width(m.shape), plan);
   }
