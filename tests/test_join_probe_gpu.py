@@ -69,3 +69,22 @@ def test_short_outputs_hold_true_pairs(npr):
     assert bool((pay[cap:] == -5).all())
     p, b = pi[:cap].cpu().numpy(), bi[:cap].cpu().numpy()
     assert (bk[b] == pk[p]).all() and (bp[b] == pay[:cap].cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("n", [2, 3, 1000, 4097, 262_144])
+@pytest.mark.parametrize("copies", [1, 2, 3, 64])
+def test_build_with_repeated_keys(n, copies):
+    """Copies of a key claim the slots behind its first one, in pairs that fill
+    up; one repeated key among different ones is noticed."""
+    rng = np.random.default_rng(n + copies)
+    bk = np.arange(n, dtype=np.int64) // copies * 7919 - n
+    if copies == 1:
+        bk[-1] = bk[0]
+    bk = bk[rng.permutation(n)]
+    bp = rng.integers(0, 2**62, n)
+    pk = np.concatenate([np.unique(bk), np.unique(bk)[:5] + 1])
+    e = oracle.join(bk, bp, pk)
+    t = rel.JoinTable(cuda(bk), cuda(bp))
+    assert t.count(cuda(pk)) == len(e[0]) == n
+    for x, y in zip(canon_join(*t.probe(cuda(pk), capacity=n)), e):
+        np.testing.assert_array_equal(x, y)
