@@ -192,7 +192,9 @@ typedef struct {
  *      rel_sketch, then the registered planner network (rel_planner_set) on
  *      its features; est_groups = max(ceil(1.25 * 2^(y0 + 1)), sample distinct
  *      keys), the variant is the network's most likely one that the
- *      descriptor supports (REL_VAR_GLOBAL: left to the rule by group count).  For one int32 / int64 key without a filter,
+ *      descriptor supports -- but REL_VAR_GLOBAL is left to the rule by group
+ *      count when the input can be partitioned or the sample's eight most
+ *      frequent keys hold 5 % of its rows.  For one int32 / int64 key without a filter,
  *      at least 2^22 rows, and a sample whose distinct keys were more than
  *      3/4 seen once (a long tail the sample cannot size), one streaming
  *      pass of a full-data HyperLogLog (4096 registers) gives est = its
@@ -333,7 +335,9 @@ rel_status rel_groupby_agg_static(const rel_groupby_desc* desc, int64_t max_grou
 /* The learned sizing rule, on the host: from a sketch and the planner
  * network's 4 outputs y (host floats: log2 of the group count, then the
  * logits of REL_VAR_SMEM, REL_VAR_GLOBAL, REL_VAR_PARTITIONED) to the
- * estimate and variant REL_PLAN_LEARNED uses.  est_groups = the smaller of
+ * estimate and the network's variant (which rel_plan_size_batched takes as it
+ * is and REL_PLAN_LEARNED unless it is REL_VAR_GLOBAL, see rel_plan_size).
+ * est_groups = the smaller of
  * n_rows and ceil(1.25 * 2^(clamp(y0, 0, 61) + 1)) (n_rows when y0 is not
  * finite), raised to the sample's distinct keys (info->ndv); variant = the
  * largest logit among the allowed variants (REL_VAR_PARTITIONED only when
