@@ -251,6 +251,9 @@ __global__ void __launch_bounds__(1024, 1) gb_gen_k(const __grid_constant__ GbPa
     __syncthreads();
   }
   unsigned long long claims = 0;
+  // Whether to look for warps whose rows are all of one group (their words are
+  // combined first): those that begin with such a chunk do
+  bool same = true;
   bool aligned = true;
   for (int c = 0; c < p.n_cols; ++c) aligned &= (uintptr_t)p.col[c] % 16 == 0;
   const int64_t CHUNK = (int64_t)blockDim.x * GEN_U;
@@ -307,9 +310,19 @@ __global__ void __launch_bounds__(1024, 1) gb_gen_k(const __grid_constant__ GbPa
       if (SET) claims += c;
     }
     if (SET) continue;
+    bool one = false;  // every row of the warp has the slot of its first
     if (SM) {
+      if (same) {
+        one = warp_same(slot[0]) && __all_sync(0xffffffffu, slot[1] == slot[0] && slot[2] == slot[0] &&
+                                                                slot[3] == slot[0]);
+        same = one || base != (int64_t)blockIdx.x * CHUNK;
+      }
+      if (one) {
+        if ((threadIdx.x & 31) == 0) reds_add(cnt + 4 * slot[0], 32 * GEN_U);
+      } else {
 #pragma unroll
-      for (int j = 0; j < GEN_U; ++j) reds_add(cnt + 4 * slot[j], 1);
+        for (int j = 0; j < GEN_U; ++j) reds_add(cnt + 4 * slot[j], 1);
+      }
     }
 #pragma unroll
     for (int j = 0; j < GEN_U; ++j)
@@ -329,7 +342,13 @@ __global__ void __launch_bounds__(1024, 1) gb_gen_k(const __grid_constant__ GbPa
       uint64_t x[GEN_U];
       agg4(p, a, r, full, x);
       if (op == REL_SUM) {
-        if (SM) {
+        if (SM && one) {
+          const uint64_t sum = warp_sum(x[0] + x[1] + x[2] + x[3]) + 32 * GEN_U * SUM_BIAS;
+          if ((threadIdx.x & 31) == 0) {
+            const uint32_t old = atoms_add(wa + 4 * slot[0], (uint32_t)sum);
+            reds_add_nz(wa + 4 * (stride + slot[0]), high_with_carry(old, sum));
+          }
+        } else if (SM) {
           uint32_t old[GEN_U];
 #pragma unroll
           for (int j = 0; j < GEN_U; ++j) old[j] = atoms_add(wa + 4 * slot[j], (uint32_t)(x[j] + SUM_BIAS));
@@ -344,7 +363,12 @@ __global__ void __launch_bounds__(1024, 1) gb_gen_k(const __grid_constant__ GbPa
         }
       } else {
         const uint64_t flip = op == REL_MIN ? MIN_FLIP : MAX_FLIP;
-        if (SM) {
+        if (SM && one) {
+          const uint64_t a = (x[0] ^ flip) > (x[1] ^ flip) ? x[0] ^ flip : x[1] ^ flip;
+          const uint64_t b = (x[2] ^ flip) > (x[3] ^ flip) ? x[2] ^ flip : x[3] ^ flip;
+          const uint64_t top = warp_max(a > b ? a : b);
+          if ((threadIdx.x & 31) == 0) reds_raise64(wa + 8 * slot[0], top, lds64(wa + 8 * slot[0]));
+        } else if (SM) {
 #pragma unroll
           for (int j = 0; j < GEN_U; ++j)
             reds_raise64(wa + 8 * slot[j], x[j] ^ flip, lds64(wa + 8 * slot[j]));

@@ -22,6 +22,8 @@
 // warp).  Runs the fused filter + aggregate shape (ShapeQ1) where its keys are
 // not all pinned (q1.cu has those) and plans with a staging ring of their own;
 // gen.cu and stream.cu have the other shapes.
+#include <type_traits>
+
 #include "groupby.cuh"
 #include "smtab.cuh"
 
@@ -1060,49 +1062,70 @@ __global__ void __launch_bounds__(GB_BLOCK, 4) gb_part_agg(const __grid_constant
   };
   bool more = next();
   if (more) start();
+  // An input in runs of rows, which the scatter keeps together: warps that begin
+  // with 32 records of one key look for the like, in a loop of its own (in the
+  // common one it is 4 to 8 % of the time of other inputs; 3e7 rows, 430000
+  // groups in runs of 64: 436 -> 346 us).
+  bool runs = false;
+  if (more) {
+#pragma unroll
+    for (int q = 0; q < PA_R; ++q) {
+      const uint64_t k = (uint64_t)rec[q].x, first = __shfl_sync(0xffffffffu, k, 0);
+      runs |= __all_sync(0xffffffffu, k == first && k != 0) != 0;
+    }
+  }
   __syncthreads();
   for (int turn = 0; more; turn ^= 1) {
     uint64_t hot = 0, hw[NA];  // the key in registers (0: none) and its words
     if (!whole) hot = frequent_key((uint64_t)rec[0].x);
 #pragma unroll
     for (int a = 0; a < NA; ++a) hw[a] = 0;
-    for (; off < len; off += STEP) {
-      uint64_t ek[PA_R], val[PA_R];
-      uint32_t slot[PA_R];
-#pragma unroll
-      for (int q = 0; q < PA_R; ++q) {
-        ek[q] = (uint64_t)rec[q].x;  // 0 past the end: a record's key is not 0
-        val[q] = (uint64_t)rec[q].y;
-      }
-      load(rec, off + STEP);
-      if (hot) {  // uniform across the warp
-        bool any = false;
+    auto rows = [&](auto in_runs) {
+      for (; off < len; off += STEP) {
+        uint64_t ek[PA_R], val[PA_R];
+        uint32_t slot[PA_R];
 #pragma unroll
         for (int q = 0; q < PA_R; ++q) {
-          if (ek[q] == hot) {
-            ek[q] = 0;
-            hw[0] += val[q];
-            hw[1] += 1;
-            if constexpr (NA == 4) {
-              const uint64_t mn = val[q] ^ MIN_FLIP, mx = val[q] ^ MAX_FLIP;
-              hw[2] = hw[2] > mn ? hw[2] : mn;
-              hw[3] = hw[3] > mx ? hw[3] : mx;
-            }
-          }
-          any |= ek[q] != 0;
+          ek[q] = (uint64_t)rec[q].x;  // 0 past the end: a record's key is not 0
+          val[q] = (uint64_t)rec[q].y;
         }
-        if (!__any_sync(0xffffffffu, any)) continue;
-      }
-      const uint32_t left = t.find(ek, 32, slot);
-      if (left) {
-        *(volatile int*)(ovf + turn) = 1;
+        load(rec, off + STEP);
+        if (hot) {  // uniform across the warp
+          bool any = false;
 #pragma unroll
-        for (int q = 0; q < PA_R; ++q)
-          if (left >> q & 1) gtab_row<S>(p, ek[q], val[q]);
+          for (int q = 0; q < PA_R; ++q) {
+            if (ek[q] == hot) {
+              ek[q] = 0;
+              hw[0] += val[q];
+              hw[1] += 1;
+              if constexpr (NA == 4) {
+                const uint64_t mn = val[q] ^ MIN_FLIP, mx = val[q] ^ MAX_FLIP;
+                hw[2] = hw[2] > mn ? hw[2] : mn;
+                hw[3] = hw[3] > mx ? hw[3] : mx;
+              }
+            }
+            any |= ek[q] != 0;
+          }
+          if (!__any_sync(0xffffffffu, any)) continue;
+        }
+        const uint32_t left = t.find(ek, 32, slot);
+        if (left) {
+          *(volatile int*)(ovf + turn) = 1;
+#pragma unroll
+          for (int q = 0; q < PA_R; ++q)
+            if (left >> q & 1) gtab_row<S>(p, ek[q], val[q]);
+        }
+        __syncwarp();
+        if constexpr (decltype(in_runs)::value)
+          t.template add_same<PA_R, 1>(slot, val);
+        else
+          t.add(slot, val);
       }
-      __syncwarp();
-      t.add(slot, val);
-    }
+    };
+    if (runs)
+      rows(std::true_type{});
+    else
+      rows(std::false_type{});
     if (hot) {  // a piece goes to the global table anyway
       Vals<NA> x;
 #pragma unroll

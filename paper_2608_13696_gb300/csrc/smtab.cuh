@@ -88,6 +88,23 @@ __device__ __forceinline__ uint32_t high_with_carry(uint32_t old, uint64_t x) {
   return h;
 }
 
+// Over the 32 lanes of a warp, all of which take part: the sum mod 2^64 (16-bit
+// halves of the low word cannot carry out of 32 bits), the largest.
+__device__ __forceinline__ uint64_t warp_sum(uint64_t x) {
+  const uint32_t a = __reduce_add_sync(0xffffffffu, (uint32_t)x & 0xFFFFu);
+  const uint32_t b = __reduce_add_sync(0xffffffffu, (uint32_t)x >> 16);
+  const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)(x >> 32));
+  return (uint64_t)a + ((uint64_t)b << 16) + ((uint64_t)c << 32);
+}
+__device__ __forceinline__ uint64_t warp_max(uint64_t x) {
+  const uint32_t h = (uint32_t)(x >> 32), top = __reduce_max_sync(0xffffffffu, h);
+  return (uint64_t)top << 32 | __reduce_max_sync(0xffffffffu, h == top ? (uint32_t)x : 0u);
+}
+// Whether every lane holds the same.
+__device__ __forceinline__ bool warp_same(uint32_t s) {
+  return __all_sync(0xffffffffu, s == __shfl_sync(0xffffffffu, s, 0));
+}
+
 // The keys of a table: buckets of two slots.
 struct KeyTab {
   static constexpr uint32_t SPARE = 32;  // slots past the table, one per lane, for idle rows
@@ -227,6 +244,54 @@ struct SmTab : KeyTab {
     }
 #pragma unroll
     for (int j = 0; j < U; ++j) reds_add_nz(hi + 4 * s[j], high_with_carry(old[j], v[j] + SUM_BIAS));
+  }
+
+  // The same for a warp whose rows may all be of one slot: those are combined
+  // first, as the adds of 32 lanes to one address take their turns (16 ns a warp
+  // and SM).  G rows of a lane that lie together are looked at together.  (Warps
+  // of two slots, as at the end of a run, cost as much in two parts as their adds
+  // do.)  All lanes of the warp.
+  template <int U, int G>
+  __device__ __forceinline__ void add_same(const uint32_t (&s)[U], const uint64_t (&v)[U]) const {
+#pragma unroll
+    for (int j = 0; j < U; j += G) {
+      uint32_t sg[G];
+      uint64_t vg[G], sum = 0, mn = 0, mx = 0;
+      bool own = true;
+      const uint32_t first = __shfl_sync(0xffffffffu, s[j], 0);
+#pragma unroll
+      for (int q = 0; q < G; ++q) {
+        sg[q] = s[j + q];
+        vg[q] = v[j + q];
+        own &= sg[q] == first;
+        sum += vg[q];
+        const uint64_t a = vg[q] ^ MIN_FLIP, b = vg[q] ^ MAX_FLIP;
+        mn = mn > a ? mn : a;
+        mx = mx > b ? mx : b;
+      }
+      // (rows without a slot are on a spare one, another in each lane)
+      if (!__all_sync(0xffffffffu, own)) {
+        add(sg, vg);
+        continue;
+      }
+      sum = warp_sum(sum) + 32 * G * SUM_BIAS;
+      if constexpr (NA == 4) {
+        mn = warp_max(mn);
+        mx = warp_max(mx);
+      }
+      if ((threadIdx.x & 31) == 0) {
+        const uint32_t old = atoms_add(lo + 4 * first, (uint32_t)sum);
+        reds_add(cnt + 4 * first, 32 * G);
+        if constexpr (NA == 4) {
+          uint64_t a, b;
+          lds128(mm + 16 * first, a, b);
+          reds_raise64(mm + 16 * first, mn, a);
+          reds_raise64(mm + 16 * first + 8, mx, b);
+        }
+        reds_add_nz(hi + 4 * first, high_with_carry(old, sum));
+      }
+      __syncwarp();
+    }
   }
 
   // The encoded words of a slot (after a barrier behind the adds).

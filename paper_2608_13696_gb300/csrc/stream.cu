@@ -315,6 +315,15 @@ __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbP
   int64_t base = (int64_t)blockIdx.x * CHUNK;
   if (base < n) ok = load(base, ek, val);
   __syncthreads();
+  // Warps that begin with 64 rows of one key -- the only one, or runs of rows
+  // -- look for the like in every chunk (3e7 rows of one key, sum and count:
+  // 146 -> 104 us; four aggregates, runs of 2500 keys 311 -> 220; 3e7 rows
+  // without runs, 100 keys: 149, 151).
+  bool same = false;
+  if (base < n) {
+    const uint64_t k = __shfl_sync(0xffffffffu, ek[0], 0);
+    same = __all_sync(0xffffffffu, ek[0] == k && ek[1] == k && ok != 0);
+  }
   for (; base < n; base += step) {
     uint64_t nek[SG_U], nval[SG_U];
     uint32_t nok = 0;
@@ -330,7 +339,10 @@ __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbP
         if (rare >> j & 1) rare_row<NA>(p, ek[j], val[j]);
     }
     __syncwarp();
-    t.add(slot, val);
+    if (same)
+      t.template add_same<SG_U, 2>(slot, val);
+    else
+      t.add(slot, val);
 #pragma unroll
     for (int j = 0; j < SG_U; ++j) {
       ek[j] = nek[j];
