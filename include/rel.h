@@ -136,6 +136,9 @@ typedef struct {
 /* Set in plan->flags by a REL_PLAN_LEARNED plan that a full-data HyperLogLog
  * sized (see rel_plan_size). */
 #define REL_PLAN_HLL_SIZED 0x20000u
+/* Set in plan->flags by REL_PLAN_SKETCH when every key of the sample is
+ * pinned: nearly every row is then expected to be. */
+#define REL_PLAN_SAMPLE_PINNED 0x40000u
 /* Test hook for the device-side wait limit, not for production use.  Set in
  * plan->flags before rel_groupby_agg: the staged kernel's consumers never hand
  * a shared-memory stage back to its producer, so once a CTA's ring has gone

@@ -664,6 +664,7 @@ void apply_sketch(const rel_sketch_info& s, int words, rel_plan* plan) {
       plan->n_hot = n;
       plan->tiny_mult = mult;
       plan->tiny_slots = (int32_t)slots;
+      if (n == s.ndv) plan->flags |= REL_PLAN_SAMPLE_PINNED;
       return;
     }
   }
@@ -702,7 +703,7 @@ rel_status set_layers(GbParams& p, const rel_plan* plan, int shape) {
              REL_E_INVALID;
     p.tiny_frozen = 1;
     p.tiny_probes = 1;
-    p.all_pinned = tiny_only;
+    p.all_pinned = tiny_only || (plan->flags & REL_PLAN_SAMPLE_PINNED);
     // at most four pinned keys, no CTA-shared layer, a shape of <= 5 words:
     // keep the accumulators in registers (dense ids in slot order).  With
     // more keys the register file costs more than it saves: 1e8 lineitem

@@ -87,7 +87,7 @@ struct GbParams {
   uint32_t tiny_mult;      // multiplier of the thread-private slot hash
   uint32_t tiny_frozen;    // 1: slots preloaded from tiny_init, no other key admitted
   uint64_t tiny_init[TINY_MAX_SLOTS];  // stored keys per slot (0 = empty)
-  uint32_t all_pinned;     // 1: a plan whose every expected group is pinned
+  uint32_t all_pinned;     // 1: every expected group, or every key of the sample, is pinned
   uint64_t tiny_dense;     // register mode: 4-bit dense id of each of <= 16 slots
   uint32_t tiny_ns;        // register mode: dense slots compiled in (4 or 8)
   int32_t req_tile, req_stages;  // staging chosen by the plan (0: automatic)

@@ -259,11 +259,24 @@ __device__ __noinline__ void rare_row(const GbParams& p, uint64_t ek, uint64_t v
   }
 }
 
+// A CTA's table into the global one (after a barrier behind the adds).
+template <int NA>
+__device__ __forceinline__ void merge_table(const GbParams& p, const SmTab<NA>& t) {
+  for (uint32_t s = threadIdx.x; s < t.slots; s += blockDim.x) {
+    const uint64_t k = t.key_of(s);
+    if (k == 0) continue;
+    uint64_t w[NA];
+    t.words(s, w);
+    global_update<NA>(p, k, w);
+  }
+}
+
 // Rows into one shared-memory table per CTA (a plan with CTA-shared slots),
 // merged into the global table at the end; rows the table has no room for go
 // to the global table one by one.  Pinned and thread-private slots of the plan
-// are not used: on a hot key the table's adds serialise over a warp's lanes
-// (15 ns a warp at worst), less than a second lookup costs every row.
+// are not used (but see PIN_TABLE_SLOTS): on a hot key the table's adds
+// serialise over a warp's lanes (15 ns a warp at worst), less than a second
+// lookup costs every row.
 constexpr int SG_U = 4;            // rows per thread per chunk
 // largest table: the rest of the SM's 256 KB is L1, through which the rows come
 // (1e8 rows, 3000 groups:
@@ -351,13 +364,7 @@ __global__ void __launch_bounds__(1024, 1) gb_smem_k(const __grid_constant__ GbP
     ok = nok;
   }
   __syncthreads();
-  for (uint32_t s = tid; s < p.smem_slots; s += B) {
-    const uint64_t k = t.key_of(s);
-    if (k == 0) continue;
-    uint64_t w[NA];
-    t.words(s, w);
-    global_update<NA>(p, k, w);
-  }
+  merge_table<NA>(p, t);
 }
 
 // Every row straight into the global table: a plan without per-CTA slots.
@@ -484,7 +491,10 @@ __host__ __device__ constexpr uint32_t pk_key_bytes() {  // per key and thread: 
 }
 constexpr uint32_t PK_HEAD = 8 * TINY_MAX_SLOTS + 8 * TINY_MAX_SLOTS * 4;  // keys, reduced words
 
-template <class KT, int NA>
+// TAB: a shared table takes the rows of other keys, for plans that expect more
+// groups than a sketch found keys; without one they go to the global table row
+// by row.
+template <class KT, int NA, bool TAB>
 __global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constant__ GbParams p) {
   extern __shared__ __align__(16) uint8_t sm[];
   uint64_t* pk = (uint64_t*)sm;  // pinned key of each slot (0: none)
@@ -492,6 +502,11 @@ __global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constan
   const uint32_t S = p.tiny_slots, B = blockDim.x, tid = threadIdx.x, tmask = S - 1;
   // [min, max pairs][sums][counts], each [slot][thread]
   const uint32_t mm = smem_u32(sm) + PK_HEAD, sum = mm + (NA == 4 ? 16 * S * B : 0), cnt = sum + 8 * S * B;
+  SmTab<NA> t;
+  if (TAB) {
+    t.bind(sm + PK_HEAD + (size_t)pk_key_bytes<NA>() * S * B, p.smem_slots);
+    t.clear();
+  }
   if (tid < TINY_MAX_SLOTS) pk[tid] = tid < S ? p.tiny_init[tid] : 0;
   for (uint32_t s = 0; s < S; ++s) {
     if (NA == 4) {
@@ -560,8 +575,31 @@ __global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constan
         }
         sts64(sum + 8 * at, o + val[j]);
         sts32(cnt + 4 * at, c + 1);
-      } else if (ok >> j & 1) {
+      } else if (!TAB && (ok >> j & 1)) {
         rare_row<NA>(p, ek[j], val[j]);
+      }
+    }
+    if constexpr (TAB) {
+      bool other = false;
+#pragma unroll
+      for (int j = 0; j < PK_U; ++j) other |= !hit[j] && (ok >> j & 1);
+      if (__any_sync(0xffffffffu, other)) {
+        uint64_t e[PK_U];
+        uint32_t slot[PK_U], rare = 0;
+#pragma unroll
+        for (int j = 0; j < PK_U; ++j) {
+          e[j] = hit[j] ? 0 : ek[j];
+          rare |= (!hit[j] && ek[j] == 0 ? 1u : 0u) << j;  // INT64_MIN
+        }
+        rare &= ok;
+        rare |= t.find(e, (int)p.shared_probes, slot);
+        if (rare) {
+#pragma unroll
+          for (int j = 0; j < PK_U; ++j)
+            if (rare >> j & 1) rare_row<NA>(p, ek[j], val[j]);
+        }
+        __syncwarp();
+        t.add(slot, val);
       }
     }
 #pragma unroll
@@ -597,6 +635,7 @@ __global__ void __launch_bounds__(PK_MAX_BLOCK, 1) gb_pin_k(const __grid_constan
     for (int a = 0; a < NA; ++a) w[a] = red[tid * NA + a];
     global_update<NA>(p, pk[tid], w);
   }
+  if (TAB) merge_table<NA>(p, t);
 }
 
 // Partitioned variant, passes 1 and 2, streaming: a CTA counts its rows per
@@ -974,10 +1013,30 @@ bool pins_fit(const GbParams& p, int na, int n_hot) {
   return p.tiny_frozen && p.tiny_slots <= 32 && n_hot <= (na == 4 ? pin_max<4>() : pin_max<2>());
 }
 
+template <class KT, int NA, bool TAB>
+rel_status launch_pin(const GbParams& p, cudaStream_t st) {
+  int block = p.n_rows > (int64_t)relhost::device_sms() * 4096 ? PK_MAX_BLOCK : 128;
+  const size_t per = p.tiny_slots * pk_key_bytes<NA>(), head = PK_HEAD + (TAB ? SmTab<NA>::bytes(p.smem_slots) : 0);
+  while (block > 128 && head + per * block > 184 * 1024) block -= 128;  // (L1)
+  return launch_rows(gb_pin_k<KT, NA, TAB>, block, head + per * block, (int64_t)block * PK_U, p, st);
+}
+
+// The largest table beside pinned keys that were all the keys of the sample
+// (a plan for at most half as many groups, though the sample has a few keys):
+// nearly every row is pinned, and three or four frequent keys meet on their
+// slots in gb_smem_k (1.45e8 rows of three Zipf(1.5) keys, four aggregates: 652
+// us there, 402 here; 3e7 rows of ten keys in runs, two aggregates: 140, 80).
+constexpr uint32_t PIN_TABLE_SLOTS = 1024;
+
 template <class KT, int NA>
 rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
   int n_hot = 0;
   for (uint32_t i = 0; i < p.tiny_slots && p.tiny_frozen; ++i) n_hot += p.tiny_init[i] != 0;
+  if (p.all_pinned && p.smem_slots && p.smem_slots <= PIN_TABLE_SLOTS && pins_fit(p, NA, n_hot)) {
+    GbParams q = p;
+    if (q.smem_slots < 256) q.smem_slots = 256;
+    return launch_pin<KT, NA, true>(q, st);
+  }
   if (p.smem_slots || (p.tiny_slots && !pins_fit(p, NA, n_hot))) {
     // 1024 resident threads per SM whatever the table's size; small inputs in
     // small CTAs, so that more SMs take part
@@ -999,12 +1058,7 @@ rel_status dispatch_layers(const GbParams& p, cudaStream_t st) {
     return launch_rows(gb_smem_k<KT, NA>, block, smem, (int64_t)block * SG_U, q, st);
   }
   const bool pin = p.tiny_frozen && p.tiny_slots;
-  if (pin && p.all_pinned) {
-    int block = p.n_rows > (int64_t)relhost::device_sms() * 4096 ? PK_MAX_BLOCK : 128;
-    const uint32_t per = p.tiny_slots * pk_key_bytes<NA>();
-    while (block > 128 && PK_HEAD + per * block > 184 * 1024) block -= 128;  // (L1)
-    return launch_rows(gb_pin_k<KT, NA>, block, PK_HEAD + (size_t)per * block, (int64_t)block * PK_U, p, st);
-  }
+  if (pin && p.all_pinned) return launch_pin<KT, NA, false>(p, st);
   if (pin) return launch_rows(gb_stream_k<KT, NA>, ST_BLOCK, stream_smem(NA), ST_BLOCK * ST_U, p, st);
   const int block = p.n_rows > (int64_t)relhost::device_sms() * 2048 ? 512 : 128;
   return launch_rows(gb_glob_k<KT, NA>, block, 0, (int64_t)block * 2, p, st);
