@@ -976,8 +976,10 @@ __device__ __forceinline__ uint64_t frequent_key(uint64_t ek) {
 //  * p.part_split: equal pieces of the record array, one per CTA, whatever
 //    partitions they touch.  For plans with fewer partitions than CTAs, whose
 //    whole partitions would leave most SMs idle (1e8 rows, 4000 groups, 16
-//    partitions: 16.8 ms in 16 CTAs).  The host sets it when the global table
-//    has a slot for every slot of the partition tables.
+//    partitions: 16.8 ms in 16 CTAs).  The host sets it where a partition has
+//    the rows for it and the global table a slot for every slot of the tables
+//    as planned: twice the groups expected.  (Tables of twice that size keep
+//    more rows at home, but no more groups than that reach the output.)
 template <int NA>
 __global__ void __launch_bounds__(GB_BLOCK, 4) gb_part_agg(const __grid_constant__ GbParams p,
                                                            const __grid_constant__ GbOut o) {

@@ -44,3 +44,23 @@ def test_results_on_both_sides(na, sketch, kind, n, groups):
     ek, ea = oracle.groupby(q)
     np.testing.assert_array_equal(k, ek)
     np.testing.assert_array_equal(a, ea)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("na", [2, 4])
+def test_low_hint_with_doubled_tables(na):
+    """Equal pieces, tables twice the planned size (many rows per partition), and
+    nearly twice the groups that were expected: they meet in the global table,
+    which has the planned slots."""
+    from gpu_util import canon_groupby, query_to_cuda
+
+    n, hint, groups = 128 * 16384 + 5, 60_000, 115_000
+    rng = np.random.default_rng(na)
+    q = oracle.kv_query(rng.integers(0, groups, n) * 31, rng.integers(-99, 99, n), ops=OPS[na])
+    qc = query_to_cuda(q)
+    p = rel.plan_groupby(qc, groups_hint=hint)
+    assert (p.part_bits, p.smem_slots, p.slots) == (7, 1024, 1 << 17)
+    k, a = canon_groupby(*rel.groupby(qc, plan=p, capacity=groups))
+    ek, ea = oracle.groupby(q)
+    np.testing.assert_array_equal(k, ek)
+    np.testing.assert_array_equal(a, ea)
