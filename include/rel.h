@@ -155,7 +155,11 @@ typedef struct {
 
 /* A plan fixes the table sizes; rows fall through thread-private slots, then
  * a CTA-shared table, then the global table (each of the first two optional),
- * so the result never depends on the plan -- only the speed does. */
+ * so the result never depends on the plan -- only the speed does.  How many
+ * layers a kernel has is its own choice: without tile_rows, key/value shapes
+ * with a CTA-shared table keep thread-private slots only when every key of the
+ * sample is pinned, and round the table up; the descriptor-driven kernel sizes
+ * its table by est_groups when either layer is wanted. */
 typedef struct {
   int64_t slots;            /* global hash-table slots (power of two >= 16)     */
   int32_t variant;          /* REL_VAR_* label of the choice                    */

@@ -495,7 +495,7 @@ rel_status run_partitioned(GbParams& p, const rel_plan* plan, int shape, const G
   uint32_t grid = 2u * (uint32_t)relhost::device_sms();
   p.fixed_grid = grid > PART_MAX_GRID ? PART_MAX_GRID : grid;
   // Tables of the aggregation pass.  At the planned load (up to 1/2) one row
-  // in ten leaves its home bucket; twice the slots make that one in 25, which
+  // in eight leaves its home bucket; twice the slots make that one in 30, which
   // pays where a partition has the records to make up for the slots it scans
   // (1e8 uniform rows, 2e6 groups, 24K records a partition: 0.83 -> 0.62 ms;
   // 2e8 Zipf rows, 9K: 1.01 -> 1.16 ms)
@@ -672,9 +672,12 @@ void apply_sketch(const rel_sketch_info& s, int words, rel_plan* plan) {
 
 // A partitioned plan's input is better off in one global table: few rows, which
 // do not make up for the partition passes' launches, and no key so frequent --
-// overall or in runs -- that its rows would queue up on one address.  (Uniform
-// keys, four aggregates, 20000 groups: 1e6 rows 42 against 93 us, 6e6 147
-// against 174, 2.5e7 550 against 434; 4000 groups cross over at 4e6 rows.)
+// overall or in runs -- that its rows would queue up on one address.  Uniform
+// keys, four aggregates, whole calls, one table against partitions: 8192 groups,
+// 1e6 rows 126 and 158 us, 2^22 rows 208 and 210, 8.4e6 306 and 276; 20000
+// groups 124 and 172, 191 and 222, 284 and 288; 200000 groups 147 and 164, 213
+// and 248, 308 and 352; 500000 groups 2^22 rows 249 and 254 (two aggregates: 95
+// to 181 against 128 to 228).  The line is where the fewest groups cross over.
 // Fewer groups than 8192 queue up on their slots, more than a quarter of the
 // rows make a table that takes longer to clear and scan.
 constexpr int64_t GLOBAL_MAX_ROWS = 1ll << 22;
@@ -704,11 +707,12 @@ rel_status set_layers(GbParams& p, const rel_plan* plan, int shape) {
     p.tiny_frozen = 1;
     p.tiny_probes = 1;
     p.all_pinned = tiny_only || (plan->flags & REL_PLAN_SAMPLE_PINNED);
-    // at most four pinned keys, no CTA-shared layer, a shape of <= 5 words:
-    // keep the accumulators in registers (dense ids in slot order).  With
-    // more keys the register file costs more than it saves: 1e8 lineitem
-    // rows with 6 pinned groups x 5 words take 1.49 ms in registers (132 of
-    // them, one 9-warp CTA per SM) and 0.96 ms in thread-private shared words
+    // The staged kernel (plans with tile_rows), at most four pinned keys, no
+    // CTA-shared layer, a shape of <= 5 words: the accumulators stay in registers
+    // (dense ids in slot order).  With more keys the register file costs more
+    // than it saves: 1e8 lineitem rows with 6 pinned groups x 5 words take 1.49 ms
+    // there in registers (132 of them, one 9-warp CTA per SM) and 0.96 ms in
+    // thread-private shared words.  Other plans run gb_q1_k and gb_pin_k.
     const bool regs_shape = shape == SHAPE_Q1 || shape == SHAPE_KV4_64 || shape == SHAPE_KV4_32 ||
                             shape == SHAPE_KV2_64 || shape == SHAPE_KV2_32;
     if (regs_shape && p.smem_slots == 0 && plan->n_hot <= 4 && p.tiny_slots <= 16) {

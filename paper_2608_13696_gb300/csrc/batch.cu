@@ -4,19 +4,21 @@
 // Most of the paper's kernel time at small scale factors sits in launches
 // too small to fill the GPU (Sec. 5.3).  Here every instance is cut into
 // tiles of blockDim x ITEMS rows; each CTA of a persistent grid (sized to the
-// resident capacity) takes the next tile from one atomic work counter, finds
-// its instance by binary search over the tiles' prefix sums, and processes
-// it.  Launch A: join builds and group-by aggregation (independent).  Launch
+// resident capacity) takes the next work item (a group-by's tiles by 32, a
+// join's probe tiles by up to 8) from one atomic work counter, finds its
+// instance in the items' prefix sums, split 32 ways a round by a warp, and
+// processes it.  Launch A: join builds and group-by aggregation (independent).  Launch
 // B: join probes (after every build) and group-by compaction (after every
 // aggregation).  The caller zeroes the counters and tables before A, so one
 // batch is one memset plus two launches, which a CUDA graph replays.
 //
 // Tables follow the single-instance kernels: open addressing on stored keys
 // key ^ 2^63 (0 = empty, INT64_MIN on a side path), zero-identity aggregate
-// words, bounded probing with an overflow flag per instance.  Probing is done
-// by W cooperating threads (W = 1, 2, 4, 8) that each read one slot of a
-// W-slot window.  Group-by instances with few groups can pre-aggregate each
-// tile in a shared-memory table and merge it into the global table.
+// words, bounded probing with an overflow flag per instance, from the key's
+// home sector of four slots.  A thread probes alone (W = 1: one sector a load)
+// or W = 2, 4 or 8 threads together, each reading one slot of a W-slot window.
+// Group-by instances whose groups fit pre-aggregate each work item in a
+// shared-memory table (smtab.cuh) and merge it into the global table.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -106,7 +108,7 @@ __device__ __forceinline__ void side_update(const BatchGb& g, BatchStatus* st, c
 
 // Global tables are walked from the first slot of the key's home sector (four
 // keys, 32 bytes): one 256-bit load shows four slots for the price of one, so
-// at most half load 97 of 100 rows end at their first load.
+// at half load 96 of 100 rows end at their first load.
 __device__ __forceinline__ uint64_t home_slot(const BatchGb& g, uint64_t ek) {
   return home_sector(ek, g.log2_slots);
 }

@@ -230,8 +230,8 @@ rel_status prepare(const rel_batch_groupby* gb, int32_t n_g, const rel_batch_joi
   long long* jbt = (long long*)at(L.off_jbt);
   long long* jpt = (long long*)at(L.off_jpt);
   jbt[0] = jpt[0] = 0;
-  // Tiles per probe work item: as many as leave every resident CTA a dozen
-  // items, at most BATCH_JOIN_SPAN (8 tiles of 64 joins of 3e5 probe rows: 712
+  // Tiles per probe work item: as many as leave an SM a dozen items (its three
+  // or more CTAs four each), at most BATCH_JOIN_SPAN (8 tiles of 64 joins of 3e5 probe rows: 712
   // us against 802 for 2 tiles; of 5e3 rows: 149 against 66).
   long long probe_tiles = 0;
   for (int i = 0; i < n_j; ++i) probe_tiles += (jn[i].n_probe + T - 1) / T;

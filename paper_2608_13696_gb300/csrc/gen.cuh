@@ -5,9 +5,7 @@
 
 namespace rel {
 
-// Whether rows of this descriptor can run on gb_gen_k (p as fill_params left
-// it, layers set).
-// Group-by: every row into a CTA-shared table of about `est` groups when that
+// Group-by (p as fill_params left it, layers set): every row into a CTA-shared table of about `est` groups when that
 // fits, merged into the global table; else straight into the global table.
 rel_status gb_launch_gen(const GbParams& p, int64_t est, cudaStream_t st);
 // Distinct qualifying keys: hdr->aux counts the keys claimed in the set

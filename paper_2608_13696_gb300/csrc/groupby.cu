@@ -1217,11 +1217,8 @@ auto with_part_shape(int shape, F&& f) {
 
 // Register-privatised kernels: shapes of at most 5 words, 4 or 8 dense slots.
 template <class F>
-auto with_regs(int shape, uint32_t ns, F&& f) {
-  auto pick = [&](auto s) {
-    using S = decltype(s);
-    return ns <= 4 ? f(BeRegs<S, 4>{}) : f(BeRegs<S, 8>{});
-  };
+auto with_regs(int shape, F&& f) {
+  auto pick = [&](auto s) { return f(BeRegs<decltype(s), 4>{}); };
   switch (shape) {
     case SHAPE_Q1: return pick(ShapeQ1{});
     case SHAPE_KV4_32: return pick(ShapeKV<int32_t, 4>{});
@@ -1276,22 +1273,6 @@ int gb_shape_width(int shape) {
   return with_shape(shape, [](auto s) { return decltype(s)::A; });
 }
 
-uint64_t gb_backend_smem_bytes(int mode, int shape, uint32_t tiny_slots, uint32_t smem_slots) {
-  if (mode == MODE_PHIST)
-    return with_part_shape(shape, [&](auto s) {
-      return BePartHist<decltype(s)>::bytes(tiny_slots, smem_slots);
-    });
-  if (mode == MODE_PSCATTER)
-    return with_part_shape(shape, [&](auto s) {
-      return BePartScatter<decltype(s)>::bytes(tiny_slots, smem_slots);
-    });
-  if (mode == MODE_TINY)
-    return with_regs(shape, 8, [&](auto be) { return decltype(be)::bytes(tiny_slots, smem_slots); });
-  return with_shape(shape, [&](auto s) {
-    return BeLayered<decltype(s)>::bytes(tiny_slots, smem_slots);
-  });
-}
-
 int gb_ctas_per_sm(const GbParams& p, int shape, int mode, bool tma) {
   if (mode == MODE_PHIST || mode == MODE_PSCATTER)
     return with_part_shape(shape, [&](auto s) {
@@ -1303,7 +1284,7 @@ int gb_ctas_per_sm(const GbParams& p, int shape, int mode, bool tma) {
                  : occupancy<S, BePartScatter<S>, false>(p);
     });
   if (mode == MODE_TINY)
-    return with_regs(shape, p.tiny_ns, [&](auto be) {
+    return with_regs(shape, [&](auto be) {
       using BE = decltype(be);
       using S = typename BE::Shape;
       return tma ? occupancy<S, BE, true>(p) : occupancy<S, BE, false>(p);
@@ -1327,7 +1308,7 @@ rel_status gb_launch_main(const GbParams& p, int shape, int mode, bool tma, cuda
                  : launch_one<S, BePartScatter<S>, false>(p, st);
     });
   if (mode == MODE_TINY)
-    return with_regs(shape, p.tiny_ns, [&](auto be) {
+    return with_regs(shape, [&](auto be) {
       using BE = decltype(be);
       using S = typename BE::Shape;
       return tma ? launch_one<S, BE, true>(p, st) : launch_one<S, BE, false>(p, st);

@@ -89,7 +89,7 @@ struct GbParams {
   uint64_t tiny_init[TINY_MAX_SLOTS];  // stored keys per slot (0 = empty)
   uint32_t all_pinned;     // 1: every expected group, or every key of the sample, is pinned
   uint64_t tiny_dense;     // register mode: 4-bit dense id of each of <= 16 slots
-  uint32_t tiny_ns;        // register mode: dense slots compiled in (4 or 8)
+  uint32_t tiny_ns;        // register mode: dense slots compiled in (4; 0: not this mode)
   int32_t req_tile, req_stages;  // staging chosen by the plan (0: automatic)
   // partitioned variant
   uint32_t part_bits;       // log2 of the partition count
@@ -145,8 +145,6 @@ rel_status gb_launch_ppass_stream(const GbParams& p, int shape, bool scatter, cu
 rel_status gb_launch_part_l2(const GbParams& p, cudaStream_t st);
 // Aggregate-array width the kernel for a shape is compiled with.
 int gb_shape_width(int shape);
-// Shared-memory bytes of the per-CTA tables (before the staging ring).
-uint64_t gb_backend_smem_bytes(int mode, int shape, uint32_t tiny_slots, uint32_t smem_slots);
 // Occupancy of a configured launch (CTAs per SM), or 0 when it cannot launch.
 int gb_ctas_per_sm(const GbParams& p, int shape, int mode, bool use_tma);
 

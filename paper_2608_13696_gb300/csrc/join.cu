@@ -11,8 +11,8 @@
 // ~64 MB) while the probe keys stream from HBM with evict-first loads and the
 // outputs leave with streaming stores.  The payload gather is fused into the
 // probe.  Slots come in pairs that fill one 32-byte sector: a key's sequence
-// starts at its home pair and one 256-bit load shows both slots, so ten of
-// eleven unique keys (load 0.48) are decided by their first load; the others
+// starts at its home pair and one 256-bit load shows both slots, so nine of
+// ten unique keys (load 0.48) are decided by their first load; the others
 // are finished in one loop per four rows, each lane on its own next row.
 #include "join.cuh"
 

@@ -298,7 +298,7 @@ rel_status mlp_forward(const void* wb, const float* p, const float* x, int batch
                        float* acts, cudaStream_t st) {
   if (batch == 0) return REL_OK;
   relhost::launch_begin(relhost::K_MLP, st);
-const int grid = (batch + FW_SAMPLES - 1) / FW_SAMPLES, most = 4 * relhost::device_sms();
+  const int grid = (batch + FW_SAMPLES - 1) / FW_SAMPLES, most = 4 * relhost::device_sms();
   mlp_fwd_k<<<grid < most ? grid : most, FW_BLOCK, 0, st>>>((const __nv_bfloat16*)wb, p, x, batch, out, acts);
   relhost::launch_end(relhost::K_MLP, st);
   return done("launch(mlp forward)");

@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(1024, 1) gb_q1_k(const __grid_constant__ GbPar
 }  // namespace
 
 bool gb_q1_eligible(const GbParams& p, int n_hot) {
-  // counts are 32 bits per thread: fewer than 2^32 rows in all is enough
+  // counts are 32 bits per thread, which sees its CTA's share of the rows: at
+  // this limit no more than 2^40 / (SMs x 128), far below 2^32
   return p.tiny_frozen && p.tiny_slots <= TINY_MAX_SLOTS && n_hot >= 1 && n_hot <= Q1_MAX_HOT &&
          p.smem_slots == 0 && p.n_rows < (1ll << 40);
 }

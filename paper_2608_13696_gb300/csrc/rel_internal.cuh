@@ -258,7 +258,7 @@ int device_sms();
 
 // Kernel ids for launch counting and event timing.
 enum KernelId : int {
-  K_GB_LAYERED = 0,
+  K_GB_LAYERED = 0,  // gb_main, gb_gen_k, gb_q1_k
   K_GB_KEYSET = 1,
   K_GB_COMPACT = 2,
   K_JOIN_BUILD = 3,
@@ -273,7 +273,7 @@ enum KernelId : int {
   K_MLP = 12,
   K_BATCH_A = 13,
   K_BATCH_B = 14,
-  K_GB_STREAM = 15,
+  K_GB_STREAM = 15,  // gb_smem_k, gb_pin_k, gb_stream_k, gb_glob_k
   K_HLL = 16,
   K_GB_PL2 = 17,
   K_COUNT_IDS = 18

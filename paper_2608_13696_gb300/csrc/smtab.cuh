@@ -10,8 +10,8 @@
 //    eight deep and more; separate 4-byte arrays use all banks (an add costs
 //    2.4 ns per warp and SM on random slots);
 //  * a key's home is a bucket of two slots, read with one 16-byte load: at
-//    half load 19 of 20 rows end there, where one-slot probing makes some lane
-//    of nearly every warp walk four slots;
+//    half load 88 of 100 keys are there (97 at a quarter), where one-slot probing
+//    makes some lane of nearly every warp walk four slots;
 //  * a thread's rows are looked up together, then updated together by
 //    straight-line code: the lanes of a warp that found their slots at
 //    different probe depths have met again before the atomics, which are
