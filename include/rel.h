@@ -200,8 +200,8 @@ typedef struct {
  *      its features; est_groups = max(ceil(1.25 * 2^(y0 + 1)), sample distinct
  *      keys), the variant is the network's most likely one that the
  *      descriptor supports -- but REL_VAR_GLOBAL is left to the rule by group
- *      count when the input can be partitioned or the sample's eight most
- *      frequent keys hold 5 % of its rows.  For one int32 / int64 key without a filter,
+ *      count unless the input cannot be partitioned, has at most 2^22 rows, and
+ *      most rows of the sample differ in their key.  For one int32 / int64 key without a filter,
  *      at least 2^22 rows, and a sample whose distinct keys were more than
  *      3/4 seen once (a long tail the sample cannot size), one streaming
  *      pass of a full-data HyperLogLog (4096 registers) gives est = its

@@ -427,10 +427,11 @@ constexpr int PART_SPLIT_BITS = 8;
 bool split_pays(int bits, int64_t n_rows, bool flat) {
   return bits <= PART_SPLIT_BITS && n_rows >> bits >= (flat ? 4000 + (200ll << bits) : 8000);
 }
-// the most groups that 256 partitions (one scatter level) take, 1024 to a
-// 2048-slot table, the same table slots in all as 512 partitions of 1024 (four
-// aggregates, 250000 groups: 2.5e7 rows 0.69 -> 0.56 ms, 1e8 2.43 -> 1.86)
-constexpr int64_t PART_ONE_LEVEL_GROUPS = 262144;
+// the most groups that 256 partitions (one scatter level) take, 1172 to a
+// 2048-slot table (four aggregates, 250000 groups: 2.5e7 rows 0.69 -> 0.56 ms,
+// 1e8 2.43 -> 1.86; 3e7 Zipf rows, 290000 groups, no sketch: 1.16 -> 0.68).  Past
+// 1024 to a table the global one has 2^20 slots, as many as 512 tables of 2048.
+constexpr int64_t PART_ONE_LEVEL_GROUPS = 300000;
 
 // Key/value plans of more than 2048 groups: the fewest slots of the global
 // table, whatever the variant.  A hint, or an estimate from a sample, may be
@@ -1149,12 +1150,16 @@ rel_status plan_groupby(const rel_groupby_desc* d, uint32_t flags, int64_t hint,
   plan->est_groups = est;
   plan->slots = (int64_t)next_pow2((uint64_t)(2 * est < 16 ? 16 : 2 * est));
   // A network that prefers the global table leaves the choice to the rule by
-  // group count where that can partition (8.4e7 rows, 7400 groups: 1.78 ms in
-  // one table, 1.12) and where the sample has frequent keys, which the rule's
-  // CTA tables keep off their one address (3e7 Zipf rows, one aggregate: 3.6 ms
-  // against 0.28).  Otherwise it is followed (2e4 rows, 6000 groups: 84 us a
-  // call, 104 with a CTA table in front).
-  if (learned == REL_VAR_GLOBAL && (p_ok || skewed(info))) learned = 0;
+  // group count, which can partition (8.4e7 rows, 7400 groups: 1.78 ms in one
+  // table, 1.12) or puts a CTA table in front for the keys that recur (1e7 rows,
+  // 1000 groups, four aggregates: 0.46 ms, 0.23; 3e7 Zipf rows, one aggregate:
+  // 3.6, 0.28).  It is followed where no CTA table can serve: few rows of mostly
+  // different keys (one aggregate, 6000 groups: 2e4 rows 84 us a call and 104 with
+  // a table in front, 1e6 rows 99 and 113; but 1e7 rows, 20000 groups, four
+  // aggregates 955 and 855).
+  if (learned == REL_VAR_GLOBAL &&
+      (p_ok || d->n_rows > GLOBAL_MAX_ROWS || 2 * info.ndv <= info.kept || skewed(info)))
+    learned = 0;
   choose_variant(forced ? forced : learned, est, d->n_rows, gb_shape_width(m.shape), p_ok,
                  sketch && !skewed(info), plan);
   if (sketch) {
