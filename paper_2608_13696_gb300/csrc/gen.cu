@@ -14,8 +14,8 @@
 //  * then one aggregate after the other: load, multiply, update the four rows'
 //    word.  Shared words are separate arrays per aggregate, sums as in
 //    smtab.cuh (two biased 32-bit halves), counts one 32-bit array.
-// Shared wavefronts and instruction issue bound it (70 % of both in ncu; 1e7 rows,
-// 3500 groups: 0.15 ms).
+// Instruction issue bounds it (60 % of the slots, 10.5 warp instructions a row;
+// 1e7 rows, 3500 groups, four aggregates: 0.15 ms).
 #include <algorithm>
 
 #include "gen.cuh"

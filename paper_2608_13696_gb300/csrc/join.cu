@@ -44,7 +44,7 @@ __device__ __forceinline__ uint64_t home_pair(uint64_t ek, int log2_slots) {
 // look at the pair: a claim that fails costs more than a look, above all in a
 // table beyond L2 or with repeated keys (whole calls on 5e6 rows, each key three
 // times: claims first 568 us, one slot a look 400, a pair 307; 10^6 different
-// keys 71, 75, 68).  Bound by the latency of the claims.
+// keys 71, 75, 68, the kernel 48 -> 45).  Bound by the latency of the claims.
 __global__ void __launch_bounds__(J_BLOCK) join_build_k(const __grid_constant__ JoinParams p,
                                                         const int64_t* __restrict__ keys,
                                                         const int64_t* __restrict__ payload,

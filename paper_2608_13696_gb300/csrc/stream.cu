@@ -9,8 +9,9 @@
 // shared-memory staging or barrier on the path.  By what the plan has:
 //  * gb_smem_k: a CTA-shared table (smtab.cuh), the global one behind it;
 //  * gb_pin_k: pinned hot keys (from the sample sketch) that are all the keys
-//    there are: a one-probe perfect-hash test, then thread-private words in
-//    shared memory (one column per thread: no atomics, no bank conflicts);
+//    there are, or all the sample had: a one-probe perfect-hash test, then
+//    thread-private words in shared memory (one column per thread: no atomics,
+//    no bank conflicts);
 //  * gb_stream_k: pinned keys and others, whose rows issue their first slot read
 //    of the global table before any is resolved, then claim or accumulate with
 //    CAS / RED atomics, bounded probing;

@@ -18,6 +18,13 @@ CASE (inputs seeded and synthetic, as in the bench):
             workload's recipe, rows divided by 8): the two persistent launches
   shard     owner split of 2e6 partial groups over 8 ranks
   hll       full-data HyperLogLog of 5e7 Zipf(1.1) keys
+  tables    2e7 uniform rows into 1000 groups through CTA tables (gb_smem_k) and
+            into 20000 through the global table alone (gb_glob_k), 2e7 Zipf rows
+            with pinned keys in front of the global table (gb_stream_k)
+  report    1e7 rows of a filtered (uint8, int32) group-by with product sums,
+            3500 groups: exact count and aggregation by descriptor (gb_gen_k)
+  staged    fused filter + group-by of 2e7 lineitem rows without a sketch (the
+            staged kernel, gb_main)
 Sizes keep every case below a few GB of device memory, with inputs above the
 129 MB L2 where the kernel streams.  Algorithmic bytes: inputs read once and
 outputs written once (16-byte records for the partition passes, 16 bytes
@@ -165,9 +172,56 @@ def case_hll(n=50_000_000):
     return {"hll": (n, "rows", 8 * n)}
 
 
+def case_tables(n=20_000_000):
+    g = torch.Generator().manual_seed(0)
+    v = torch.randint(-10**6, 10**6, (n,), generator=g).cuda()
+
+    def run(groups, flags):
+        k = torch.randint(0, groups, (n,), generator=g).cuda() * 1_000_003
+        q = kv_query(k, v)
+        rel.groupby(q, plan=rel.plan_groupby(q, flags=flags, groups_hint=groups))
+
+    run(1000, 0)
+    run(20_000, rel.plan_force(rel.VAR_GLOBAL))
+    import synth
+
+    zk, zv = synth.zipf_kv(n, seed=0)
+    q = kv_query(_cuda(zk), _cuda(zv))
+    p = rel.plan_groupby(q, flags=rel.PLAN_SKETCH | rel.plan_force(rel.VAR_GLOBAL),
+                         groups_hint=2_000_000)
+    rel.groupby(q, plan=p)
+    return {"gb_stream": (n, "rows", 16 * n)}
+
+
+def case_report(n=10_000_000, stores=700):
+    g = torch.Generator().manual_seed(0)
+
+    def col(lo, hi, dtype=torch.int64):
+        return torch.randint(lo, hi + 1, (n,), generator=g).to(dtype).cuda()
+
+    q = {"cols": [col(0, 4, torch.uint8), col(1, stores, torch.int32), col(0, 364, torch.int32),
+                  col(1, 500_000), col(0, 30)], "keys": [0, 1],
+         "preds": [(2, 30, 329), (3, 1_000, 499_000)],
+         "aggs": [("sum", 3, [(4, 100, -1)]), ("min", 3, []), ("max", 3, []), ("count", 3, [])]}
+    rel.groupby(q, plan=rel.plan_groupby(q, flags=rel.PLAN_EXACT))
+    return {"gb_gen_set": (n, "rows", 17 * n), "gb_gen": (n, "rows", 25 * n)}
+
+
+def case_staged(n=20_000_000):
+    import synth
+
+    from .workloads import lineitem_query
+
+    q = lineitem_query(synth.lineitem(n, seed=0))
+    q["cols"] = [_cuda(c) for c in q["cols"]]
+    rel.groupby(q, plan=rel.plan_groupby(q, groups_hint=6))
+    return {"gb_main": (n, "rows", sum(c.nbytes for c in q["cols"]))}
+
+
 CASES = {"distinct": case_distinct, "part": case_part, "stream": case_stream,
          "join": case_join, "lineitem": case_lineitem, "mlp": case_mlp, "batch": case_batch,
-         "shard": case_shard, "hll": case_hll}
+         "shard": case_shard, "hll": case_hll, "tables": case_tables, "report": case_report,
+         "staged": case_staged}
 
 
 def main(argv) -> None:
